@@ -71,6 +71,7 @@ enum KernelKind : int {
     KIND_COL_SD = 3,   // power of two, element-contiguous in (ZYX load), strided out
     KIND_ROW_R2C = 4,  // power-of-two half length, X-stage real-to-complex
     KIND_ROW_C2R = 5,  // power-of-two half length, X-stage complex-to-real
+    KIND_FIX64 = 6,    // FP64 data, 64-bit block fixed-point arithmetic (p3_fix64.cuh)
 };
 
 enum StageOp : int {
@@ -135,6 +136,7 @@ struct StageArgs {
     size_t smem;       // dynamic shared memory bytes
     int threads;       // B * tpl
     int kern;          // KernelKind
+    int fix;           // KIND_FIX64: which of its kernels (32 fx::Kind + largest radix)
     // 1: tensor-core split-precision kernel (p3_tc.cu)
     int tc;
     // 1: TMA-staged ZYX-store column kernel (input tile by tensor copies);
@@ -178,6 +180,28 @@ cudaError_t launch_stage_f32(const StageArgs& a, cudaStream_t s);
 cudaError_t launch_stage_f64(const StageArgs& a, cudaStream_t s);
 // One-time kernel attribute set-up for the current device (max dynamic smem).
 cudaError_t prepare_kernels();
+
+// FP64 fixed-point kernels (p3_fix64.cu).  a.tw and a.tw2 hold twiddles in
+// fixed point there: {re high, re low, im high, im low} of exp(-2 pi i k / n)
+// 2^60, the low halves signed.
+//
+// Threads per line of a radix sequence in the kernels of largest radix cap
+// (8, 10 or 16); 0: more than a CTA has.
+int fix64_threads(int n, int npass, const int* rad, int cap);
+// Tile shape of a stage whose radices and a.fix (the cap) are set (shrink halves the lines per
+// CTA that many times; false when none is left).
+bool fix64_configure(StageArgs& a, int shrink);
+cudaError_t fix64_prepare();
+cudaError_t fix64_launch(const StageArgs& a, cudaStream_t s);
+// FP64 plans of at most this many points (Nx Ny Nz) take them.  Their results
+// are nearer to the exact transform than the double-arithmetic kernels' at
+// every size, but they are other roundings: in larger volumes the double
+// kernels' own error in the bins beside a strong wave (up to 1.3e-12 of the
+// spectrum's typical bin at 512^3; 4.7e-13 once in fifty runs at 250 x 256 x
+// 250) exceeds the agreement with earlier results that perf/cases.py holds
+// outputs to (4.4e-13).  At 243 x 250 x 180 the largest of ten runs was
+// 2.4e-13.
+constexpr double kFix64MaxPoints = 12582912.0;
 
 // Power-of-two specialised kernels (p3_pow2.cu): configure a stage for them
 // (returns false when none applies), set them up, launch one stage.

@@ -842,6 +842,7 @@ cudaError_t launch_stage_f32(const StageArgs& a, cudaStream_t s)
 }
 cudaError_t launch_stage_f64(const StageArgs& a, cudaStream_t s)
 {
+    if (a.kern == KIND_FIX64) return fix64_launch(a, s);
     return a.kern != KIND_GENERIC ? pow2_launch(a, false, s) : launch_stage<double>(a, s);
 }
 
@@ -853,6 +854,8 @@ cudaError_t prepare_kernels()
     e = cudaFuncSetAttribute(stage_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
     e = pow2_prepare();
+    if (e != cudaSuccess) return e;
+    e = fix64_prepare();
     if (e != cudaSuccess) return e;
     return tc_prepare();
 }

@@ -46,7 +46,7 @@ struct Stage {
 };
 
 struct TableKey {
-    int kind;  // 0 roots, 1 chirp, 2 bhat
+    int kind;  // 0 roots, 1 chirp, 2 bhat, 3 row-style roots, 4 fixed-point roots
     long long n, m;
     bool operator<(const TableKey& o) const
     {
@@ -90,9 +90,9 @@ namespace {
 
 const long double kPi = 3.141592653589793238462643383279502884L;
 
-// exp(-2 pi i k / n) in FP64: the angle is reduced exactly to octant o and an
-// offset x in [0, pi/4] before cosl/sinl, then rotated back by symmetry.
-std::complex<double> unit_root(long long k, long long n)
+// exp(-2 pi i k / n): the angle is reduced exactly to octant o and an offset
+// x in [0, pi/4] before cosl/sinl, then rotated back by symmetry.
+std::complex<long double> unit_root_l(long long k, long long n)
 {
     k %= n;
     if (k < 0) k += n;
@@ -118,7 +118,33 @@ std::complex<double> unit_root(long long k, long long n)
         default: c = cy; s = -sy; break;
         }
     }
-    return std::complex<double>((double)c, -(double)s);
+    return std::complex<long double>(c, -s);
+}
+// the same rounded to FP64
+std::complex<double> unit_root(long long k, long long n)
+{
+    const std::complex<long double> w = unit_root_l(k, n);
+    return std::complex<double>((double)w.real(), (double)w.imag());
+}
+
+// The same times 2^60 for the FP64 fixed-point kernels: the parts' high and
+// (signed) low 32-bit halves, in the 16 bytes of one table entry.
+std::complex<double> fixed_root(long long k, long long n)
+{
+    const std::complex<long double> w = unit_root_l(k, n);
+    int h[4];
+    const long double part[2] = {w.real(), w.imag()};
+    for (int i = 0; i < 2; ++i) {
+        long long q = llrintl(part[i] * 1152921504606846976.0L);
+        if ((int)(unsigned)(unsigned long long)q == INT32_MIN) ++q;  // so that the low half has a negative
+        const int lo = (int)(unsigned)(unsigned long long)q;
+        h[2 * i] = (int)((q - lo) >> 32);
+        h[2 * i + 1] = lo;
+    }
+    std::complex<double> e;
+    static_assert(sizeof(e) == sizeof(h), "one entry");
+    memcpy(&e, h, sizeof(h));
+    return e;
 }
 
 // In-place iterative radix-2 DFT (exp(-2 pi i ...)) in long double, for the
@@ -156,7 +182,9 @@ void host_dft_pow2(std::vector<std::complex<long double>>& a)
 // register butterflies 6 .. 28, ties going to the one whose smallest radix is
 // largest, largest radix first.  Returns false when n has a prime factor
 // above 7.
-bool factor(int n, std::vector<int>& rad, bool composite = false)
+// cap > 0 (FP64 fixed-point stages): as composite = true, for every smooth n,
+// with no radix above cap.
+bool factor(int n, std::vector<int>& rad, bool composite = false, int cap = 0)
 {
     rad.clear();
     int m = n;
@@ -166,7 +194,7 @@ bool factor(int n, std::vector<int>& rad, bool composite = false)
     while (m > 1 && m % 5 == 0) { m /= 5; ++e5; }
     while (m > 1 && m % 7 == 0) { m /= 7; ++e7; }
     if (m != 1) return false;
-    if (composite && e3 + e5 + e7 > 0) {
+    if (cap > 0 || (composite && e3 + e5 + e7 > 0)) {
         // radices as exponent vectors (2, 3, 5, 7)
         static const int kRad[][5] = {
             {28, 2, 0, 0, 1}, {27, 0, 3, 0, 0}, {25, 0, 0, 2, 0}, {24, 3, 1, 0, 0}, {21, 0, 1, 0, 1},
@@ -186,7 +214,7 @@ bool factor(int n, std::vector<int>& rad, bool composite = false)
             Best r{1 << 30, 0, {}};
             for (const auto& k : kRad) {
                 if (k[1] > a || k[2] > b || k[3] > c || k[4] > d) continue;
-                if (k[0] > p3::kMaxCompositeRadix && k[0] != 16) continue;
+                if (cap > 0 ? k[0] > cap : k[0] > p3::kMaxCompositeRadix && k[0] != 16) continue;
                 Best t = best(a - k[1], b - k[2], c - k[3], d - k[4]);
                 const int passes = t.passes + 1, minr = std::min(t.minr, k[0]);
                 if (passes < r.passes || (passes == r.passes && minr > r.minr)) {
@@ -278,6 +306,14 @@ size_t roots_table(TableSet& T, long long n)
     return T.add(TableKey{0, n, 0}, std::move(v));
 }
 
+// the same for the FP64 fixed-point kernels
+size_t fixed_roots_table(TableSet& T, long long n)
+{
+    std::vector<std::complex<double>> v((size_t)n);
+    for (long long k = 0; k < n; ++k) v[(size_t)k] = fixed_root(k, n);
+    return T.add(TableKey{4, n, 0}, std::move(v));
+}
+
 // Per-pass twiddles of a power-of-two line of n points with E values per
 // thread, laid out for row-style lanes (see rtw_off in p3_pow2.cuh): pass
 // p >= 1 (NS = the product of the earlier radices, radix R, step n/(NS R))
@@ -334,9 +370,53 @@ struct Pending {
     size_t tw = 0, tw2 = 0, chirp = 0, bhat = 0, twm = 0, twr = 0;
 };
 
+// Which form of the FP64 fixed-point kernels a stage of nlines lines of n
+// points takes (their largest radix 8, 10 or 16; 0: none) and its radices.
+// rows: the X stage.  The weights are relative times fitted to cubes of 128 to
+// 256 and mixed grids: the one-butterfly forms (8, 10)
+// cost 0.16 + 0.28 per pass, the 16-value form 0.05 + 0.45.  For example, Y
+// lines of 200 points take 70 us in three passes of the first and 96 in three
+// of the second; 256 points 164 us in three (8 8 4) and 117 in two (16 16);
+// 250 points 125 us in three (10 5 5) against 158.  A one-butterfly form
+// whose narrowest pass leaves most of a line's threads idle (192 points:
+// 8 6 4) or whose tiles are two or one lines wide (1024 points: 233 against
+// 155 us) loses its advantage.  Stages of at most 2^18 values are bound by the
+// chain of one pass: form 8 (32^3 pair 35 us against 68 us in form 16).
+int fixed_form(long long nlines, int n, bool rows, std::vector<int>& rad)
+{
+    static const int caps[3] = {8, 10, 16};
+    int pick = -1;
+    double best = 0.0;
+    for (int i = 0; i < 3; ++i) {
+        std::vector<int> r;
+        const int tpl = factor(n, r, true, caps[i]) ? p3::fix64_threads(n, (int)r.size(), r.data(), caps[i]) : 0;
+        if (!tpl) continue;
+        const double p = (double)r.size();
+        double cost;
+        if (caps[i] == 16) {
+            cost = (0.05 + 0.45 * p) * (rows ? 1.15 : 1.0);
+            if (std::find(r.begin(), r.end(), 15) != r.end()) cost *= 1.08;
+        } else {
+            const double used = (double)(n / r[0]) / tpl;  // threads busy in the pass of the largest radix
+            cost = (0.16 + 0.28 * p) * (used < 0.45 ? 1.5 : used <= 0.6 ? 1.2 : 1.0) *
+                   (tpl > 128 ? 1.65 : tpl > 64 ? 1.2 : tpl == 64 && (n & (n - 1)) == 0 ? 1.2 : 1.0);
+            if (caps[i] == 8 && nlines * n <= (1LL << 18)) cost = 0.0;
+        }
+        if (pick < 0 || cost < best) {
+            pick = i;
+            best = cost;
+            rad = r;
+        }
+    }
+    if (pick < 0) rad.clear();
+    return pick < 0 ? 0 : caps[pick];
+}
+
 // Line-FFT set-up: native radices over nfft, else Bluestein over m.
+// fixed: the FP64 fixed-point kernels with that radix sequence.
 // Returns P3_ERR_UNSUPPORTED for lines beyond the shared-memory limit.
-p3_status line_setup(StageArgs& a, Pending& pend, TableSet& T, int twn_native, bool composite)
+p3_status line_setup(StageArgs& a, Pending& pend, TableSet& T, int twn_native, bool composite,
+                     const std::vector<int>& fixed)
 {
     std::vector<int> rad;
     a.blue = 0;
@@ -345,6 +425,13 @@ p3_status line_setup(StageArgs& a, Pending& pend, TableSet& T, int twn_native, b
     a.m = 0;
     if (a.nfft <= 1) {
         a.tpl = 1;
+        return P3_OK;
+    }
+    if (!fixed.empty()) {
+        a.npass = (int)fixed.size();
+        for (int i = 0; i < a.npass; ++i) a.rad[i] = fixed[i];
+        a.twn = twn_native;
+        pend.tw = fixed_roots_table(T, twn_native) + 1;
         return P3_OK;
     }
     if (factor(a.nfft, rad, composite)) {
@@ -400,8 +487,12 @@ void generic_tile_setup(StageArgs& a, size_t csize, size_t cap = P3_GEN_SMEM_CAP
     a.tma = 0;
 }
 
-void tile_setup(StageArgs& a, size_t csize, unsigned flags)
+void tile_setup(StageArgs& a, size_t csize, unsigned flags, bool fixed)
 {
+    if (fixed) {
+        p3::fix64_configure(a, 0);
+        return;
+    }
     generic_tile_setup(a, csize);
     p3::pow2_configure(a, csize, !(flags & P3_FLAG_NO_TMA));
     if (flags & P3_FLAG_TC_SPLIT) p3::tc_configure(a, csize);
@@ -423,9 +514,17 @@ const char* op_name(int op)
     }
 }
 
-const char* kern_name(int k, int tc, int tma = 0)
+const char* kern_name(const StageArgs& a)
 {
-    if (tc) return "tc_split_col";
+    const int k = a.kern, tma = a.tma;
+    if (k == p3::KIND_FIX64) {
+        // power-of-two lengths keep the names of their FP32 counterparts
+        if (a.nfft < 64 || (a.nfft & (a.nfft - 1))) return "fix64";
+        if (a.op == p3::OP_R2C_HALF) return "pow2_row_r2c_fix64";
+        if (a.op == p3::OP_C2R_HALF) return "pow2_row_c2r_fix64";
+        return a.out_elem_fast ? "pow2_col_zyx_store_fix64" : a.in_elem_fast ? "pow2_col_zyx_load_fix64" : "pow2_col_fix64";
+    }
+    if (a.tc) return "tc_split_col";
     if (tma == 2) return "pow2_zrow_bulk";
     if (tma) return "pow2_col_zyx_store_tma";
     switch (k) {
@@ -559,6 +658,11 @@ static p3_status tune(p3_plan P, std::vector<Stage> (&unfused)[3], std::string& 
 // of its factorisation and tile heights B, B / 2, B / 4 on temporary
 // buffers, and keep the fastest.  Any order is the same DFT with the same
 // root table; only rounding differs.
+static bool tunable(const Stage& st)
+{
+    return !st.fused && (st.a.kern == p3::KIND_GENERIC || st.a.kern == p3::KIND_FIX64) && !st.a.blue &&
+           st.a.op != p3::OP_COPY && st.a.npass > 1;
+}
 static p3_status tune_generic(p3_plan P, std::string& report)
 {
     const size_t rowr = P->padded ? 2 * (size_t)P->H : (size_t)P->nx;
@@ -568,8 +672,7 @@ static p3_status tune_generic(p3_plan P, std::string& report)
     bool any = false;
     for (int d = 0; d < 2; ++d)
         for (const Stage& st : P->st[d])
-            if (!st.fused && st.a.kern == p3::KIND_GENERIC && !st.a.blue && st.a.op != p3::OP_COPY && st.a.npass > 1)
-                any = true;
+            if (tunable(st)) any = true;
     if (!any) return P3_OK;
     void* buf[3] = {NULL, NULL, NULL};
     cudaStream_t sm = NULL;
@@ -586,7 +689,7 @@ static p3_status tune_generic(p3_plan P, std::string& report)
         for (size_t si = 0; si < P->st[d].size() && rc == P3_OK; ++si) {
             Stage& st = P->st[d][si];
             StageArgs& a0 = st.a;
-            if (st.fused || a0.kern != p3::KIND_GENERIC || a0.blue || a0.op == p3::OP_COPY || a0.npass <= 1) continue;
+            if (!tunable(st)) continue;
             // candidate radix orders: as factored, reversed, ascending, and
             // each rotation of the factored order
             std::vector<std::vector<int>> orders;
@@ -611,9 +714,13 @@ static p3_status tune_generic(p3_plan P, std::string& report)
                 for (int shrink = 0; shrink < 3 && rc == P3_OK; ++shrink) {
                     StageArgs a = a0;
                     for (size_t k = 0; k < o.size(); ++k) a.rad[k] = o[k];
-                    generic_tile_setup(a, P->csize);
-                    if ((a.B >> shrink) < 1) break;
-                    if (shrink) {
+                    if (a0.kern == p3::KIND_FIX64) {
+                        if (!p3::fix64_configure(a, shrink)) break;
+                    } else {
+                        generic_tile_setup(a, P->csize);
+                        if ((a.B >> shrink) < 1) break;
+                    }
+                    if (shrink && a0.kern == p3::KIND_GENERIC) {
                         a.B >>= shrink;
                         const bool elem = a.in_elem_fast || a.out_elem_fast;
                         a.LDB = (elem && (a.B % 2 == 0)) ? a.B + 1 : a.B;
@@ -739,6 +846,9 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
                 : ttype[2] == P3_SINE ? 2.0 * (nz + 1)
                                       : 1.0;
 
+    // FP64 plans of up to kFix64MaxPoints points run in 64-bit fixed point
+    const bool fixed = prec == P3_F64 && (double)nx * ny * nz <= p3::kFix64MaxPoints;
+
     TableSet T;
     std::vector<Pending> pend[3];
     p3_status rc = P3_OK;
@@ -768,15 +878,20 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
     auto push = [&](int dir, StageArgs a, int src, int dst, const char* name, double bytes, int twn) {
         Pending pd;
         if (rc != P3_OK) return;
+        // the fixed-point radix sequence (empty: the line does not run there)
+        std::vector<int> fx;
+        if (fixed && a.op != p3::OP_COPY && a.nfft > 1 && a.nfft <= p3::kMaxLine) {
+            a.fix = fixed_form(a.nlines, a.nfft, a.op != p3::OP_C2C && a.op != p3::OP_DCT1 && a.op != p3::OP_DST1, fx);
+        }
         if (a.op == p3::OP_R2C_HALF || a.op == p3::OP_C2R_HALF) {
-            pd.tw2 = roots_table(T, NX) + 1;
+            pd.tw2 = (fx.empty() ? roots_table(T, NX) : fixed_roots_table(T, NX)) + 1;
         }
         if (a.op != p3::OP_COPY) {
-            rc = line_setup(a, pd, T, twn, prec == P3_F32 && P3_GEN_COMPOSITE);
+            rc = line_setup(a, pd, T, twn, prec == P3_F32 && P3_GEN_COMPOSITE, fx);
             if (rc != P3_OK) return;
             // row-style twiddles for power-of-two lines (E as the row kernels take it)
             const long long n = a.nfft;
-            if (!a.blue && n >= 64 && n <= 4096 && (n & (n - 1)) == 0) {
+            if (fx.empty() && !a.blue && n >= 64 && n <= 4096 && (n & (n - 1)) == 0) {
                 const int E = (prec == P3_F32 && n >= 512 && n <= 2048) ? 32 : 16;
                 const bool half = a.op == p3::OP_R2C_HALF || a.op == p3::OP_C2R_HALF;
                 pd.twr = row_tw_table(T, n, E, half ? 2 * n : n) + 1;
@@ -786,7 +901,7 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
             a.nfft = a.n_in;  // slots per line; no FFT passes
             a.npass = 0;
         }
-        tile_setup(a, P->csize, flags);
+        tile_setup(a, P->csize, flags, !fx.empty());
         Stage s;
         s.a = a; s.src = src; s.dst = dst; s.name = name; s.bytes = bytes;
         s.fused = false;
@@ -917,7 +1032,7 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
                 z.a.out = ws_lines;
             }
             // same kernel kind; the new maps can admit a TMA-fed variant
-            if (z.a.kern != p3::KIND_GENERIC) p3::pow2_configure(z.a, P->csize, !(flags & P3_FLAG_NO_TMA));
+            if (z.a.kern != p3::KIND_GENERIC && z.a.kern != p3::KIND_FIX64) p3::pow2_configure(z.a, P->csize, !(flags & P3_FLAG_NO_TMA));
         }
     }
     const bool any_fused = fuse_at[0] >= 0 || fuse_at[1] >= 0 || fuse_at[2] >= 0;
@@ -950,8 +1065,7 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
                 float v[2] = {(float)T.vals[i].real(), (float)T.vals[i].imag()};
                 memcpy(&host[i * 8], v, 8);
             } else {
-                double v[2] = {T.vals[i].real(), T.vals[i].imag()};
-                memcpy(&host[i * 16], v, 16);
+                memcpy(&host[i * 16], &T.vals[i], 16);  // doubles or fixed-point entries
             }
         }
         cudaError_t ce = cudaMalloc(&P->dtab, bytes);
@@ -1094,7 +1208,21 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
                 continue;
             }
             std::string rs;
-            if (a.kern != p3::KIND_GENERIC) {
+            if (a.kern == p3::KIND_FIX64) {
+                // composite register butterflies as the native radices they are made of
+                for (int i = 0; i < a.npass; ++i) {
+                    switch (a.rad[i]) {
+                    case 6: rs += "2x3"; break;
+                    case 9: rs += "3x3"; break;
+                    case 10: rs += "2x5"; break;
+                    case 12: rs += "4x3"; break;
+                    case 14: rs += "2x7"; break;
+                    case 15: rs += "3x5"; break;
+                    default: rs += std::to_string(a.rad[i]); break;
+                    }
+                    if (i + 1 < a.npass) rs += "x";
+                }
+            } else if (a.kern != p3::KIND_GENERIC) {
                 // power-of-two kernels: radix E = nfft / tpl while it divides, then the rest
                 const int E = a.nfft / a.tpl;
                 int n = a.nfft;
@@ -1115,7 +1243,7 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
             snprintf(line, sizeof(line),
                      "%s %s kernel=%s op=%s nfft=%d%s radices=%s lines=%lld B=%d LDB=%d tpl=%d threads=%d "
                      "smem=%zu bytes=%.0f\n",
-                     d == 0 ? "fwd" : "bwd", s.name, kern_name(a.kern, a.tc, a.tma), op_name(a.op), a.nfft,
+                     d == 0 ? "fwd" : "bwd", s.name, kern_name(a), op_name(a.op), a.nfft,
                      a.blue ? (" bluestein_m=" + std::to_string(a.m)).c_str() : "", rs.c_str(), a.nlines, a.B,
                      a.LDB, a.tpl, a.threads, a.smem, s.bytes);
             P->desc += line;
