@@ -100,15 +100,9 @@ bool fix64_configure(StageArgs& a, int shrink)
     return true;
 }
 
-cudaError_t fix64_prepare()
+cudaError_t fix64_prepare(const StageArgs& a)
 {
-    for (int k = fx::K_CC; k <= fx::K_CP; ++k)
-        for (int cap : {8, 10, 16}) {
-            const cudaError_t e = cudaFuncSetAttribute(pick(k, cap), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       110 * 1024);
-            if (e != cudaSuccess) return e;
-        }
-    return cudaSuccess;
+    return cudaFuncSetAttribute(pick(a.fix >> 5, a.fix & 31), cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024);
 }
 
 cudaError_t fix64_launch(const StageArgs& a0, cudaStream_t st)

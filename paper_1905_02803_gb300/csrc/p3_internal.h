@@ -72,6 +72,7 @@ enum KernelKind : int {
     KIND_ROW_R2C = 4,  // power-of-two half length, X-stage real-to-complex
     KIND_ROW_C2R = 5,  // power-of-two half length, X-stage complex-to-real
     KIND_FIX64 = 6,    // FP64 data, 64-bit block fixed-point arithmetic (p3_fix64.cuh)
+    KIND_LINE32 = 7,   // FP32, smooth lengths, register passes in place (p3_line32.cuh)
 };
 
 enum StageOp : int {
@@ -136,7 +137,7 @@ struct StageArgs {
     size_t smem;       // dynamic shared memory bytes
     int threads;       // B * tpl
     int kern;          // KernelKind
-    int fix;           // KIND_FIX64: which of its kernels (32 fx::Kind + largest radix)
+    int fix;           // KIND_FIX64: which of its kernels (32 fx::Kind + largest radix); KIND_LINE32: l32::Kind
     // 1: tensor-core split-precision kernel (p3_tc.cu)
     int tc;
     // 1: TMA-staged ZYX-store column kernel (input tile by tensor copies);
@@ -178,8 +179,10 @@ inline void generic_consts(StageArgs& a)
 // Launch one stage (defined in p3_kernels.cu).  Returns the launch error.
 cudaError_t launch_stage_f32(const StageArgs& a, cudaStream_t s);
 cudaError_t launch_stage_f64(const StageArgs& a, cudaStream_t s);
-// One-time kernel attribute set-up for the current device (max dynamic smem).
+// One-time kernel attribute set-up for the current device (max dynamic smem):
+// of the kernels that any plan may take, and of a configured stage's own.
 cudaError_t prepare_kernels();
+cudaError_t prepare_stage(const StageArgs& a);
 
 // FP64 fixed-point kernels (p3_fix64.cu).  a.tw and a.tw2 hold twiddles in
 // fixed point there: {re high, re low, im high, im low} of exp(-2 pi i k / n)
@@ -191,7 +194,7 @@ int fix64_threads(int n, int npass, const int* rad, int cap);
 // Tile shape of a stage whose radices and a.fix (the cap) are set (shrink halves the lines per
 // CTA that many times; false when none is left).
 bool fix64_configure(StageArgs& a, int shrink);
-cudaError_t fix64_prepare();
+cudaError_t fix64_prepare(const StageArgs& a);
 cudaError_t fix64_launch(const StageArgs& a, cudaStream_t s);
 // FP64 plans of at most this many points (Nx Ny Nz) take them.  Their results
 // are nearer to the exact transform than the double-arithmetic kernels' at
@@ -202,6 +205,13 @@ cudaError_t fix64_launch(const StageArgs& a, cudaStream_t s);
 // outputs to (4.4e-13).  At 243 x 250 x 180 the largest of ten runs was
 // 2.4e-13.
 constexpr double kFix64MaxPoints = 12582912.0;
+
+// FP32 line kernels of smooth lengths (p3_line32.cu): configure a stage whose
+// radices are set (false when none applies; shrink halves the lines per CTA
+// that many times), set them up, launch one stage.
+bool line32_configure(StageArgs& a, int shrink);
+cudaError_t line32_prepare(const StageArgs& a);
+cudaError_t line32_launch(const StageArgs& a, cudaStream_t s);
 
 // Power-of-two specialised kernels (p3_pow2.cu): configure a stage for them
 // (returns false when none applies), set them up, launch one stage.

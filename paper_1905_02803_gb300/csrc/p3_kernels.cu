@@ -838,12 +838,18 @@ cudaError_t batch_launch(const BatchLaunch& b, int grid, size_t smem, cudaStream
 cudaError_t launch_stage_f32(const StageArgs& a, cudaStream_t s)
 {
     if (a.tc) return tc_launch(a, s);
+    if (a.kern == KIND_LINE32) return line32_launch(a, s);
     return a.kern != KIND_GENERIC ? pow2_launch(a, true, s) : launch_stage<float>(a, s);
 }
 cudaError_t launch_stage_f64(const StageArgs& a, cudaStream_t s)
 {
     if (a.kern == KIND_FIX64) return fix64_launch(a, s);
     return a.kern != KIND_GENERIC ? pow2_launch(a, false, s) : launch_stage<double>(a, s);
+}
+
+cudaError_t prepare_stage(const StageArgs& a)
+{
+    return a.kern == KIND_FIX64 ? fix64_prepare(a) : a.kern == KIND_LINE32 ? line32_prepare(a) : cudaSuccess;
 }
 
 cudaError_t prepare_kernels()
@@ -854,8 +860,6 @@ cudaError_t prepare_kernels()
     e = cudaFuncSetAttribute(stage_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
     e = pow2_prepare();
-    if (e != cudaSuccess) return e;
-    e = fix64_prepare();
     if (e != cudaSuccess) return e;
     return tc_prepare();
 }

@@ -494,7 +494,7 @@ void tile_setup(StageArgs& a, size_t csize, unsigned flags, bool fixed)
         return;
     }
     generic_tile_setup(a, csize);
-    p3::pow2_configure(a, csize, !(flags & P3_FLAG_NO_TMA));
+    if (!p3::pow2_configure(a, csize, !(flags & P3_FLAG_NO_TMA)) && csize == 8) p3::line32_configure(a, 0);
     if (flags & P3_FLAG_TC_SPLIT) p3::tc_configure(a, csize);
 }
 
@@ -533,6 +533,7 @@ const char* kern_name(const StageArgs& a)
     case p3::KIND_COL_SD: return "pow2_col_zyx_load";
     case p3::KIND_ROW_R2C: return "pow2_row_r2c";
     case p3::KIND_ROW_C2R: return "pow2_row_c2r";
+    case p3::KIND_LINE32: return "line32";
     default: return "generic";
     }
 }
@@ -660,7 +661,8 @@ static p3_status tune(p3_plan P, std::vector<Stage> (&unfused)[3], std::string& 
 // root table; only rounding differs.
 static bool tunable(const Stage& st)
 {
-    return !st.fused && (st.a.kern == p3::KIND_GENERIC || st.a.kern == p3::KIND_FIX64) && !st.a.blue &&
+    return !st.fused && (st.a.kern == p3::KIND_GENERIC || st.a.kern == p3::KIND_FIX64 || st.a.kern == p3::KIND_LINE32) &&
+           !st.a.blue &&
            st.a.op != p3::OP_COPY && st.a.npass > 1;
 }
 static p3_status tune_generic(p3_plan P, std::string& report)
@@ -716,6 +718,8 @@ static p3_status tune_generic(p3_plan P, std::string& report)
                     for (size_t k = 0; k < o.size(); ++k) a.rad[k] = o[k];
                     if (a0.kern == p3::KIND_FIX64) {
                         if (!p3::fix64_configure(a, shrink)) break;
+                    } else if (a0.kern == p3::KIND_LINE32) {
+                        if (!p3::line32_configure(a, shrink)) break;
                     } else {
                         generic_tile_setup(a, P->csize);
                         if ((a.B >> shrink) < 1) break;
@@ -1056,6 +1060,13 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
         delete P;
         return P3_ERR_CUDA;
     }
+    for (int d = 0; d < 3; ++d)
+        for (const Stage& s : P->st[d])
+            if (p3::prepare_stage(s.a) != cudaSuccess) {
+                cudaGetLastError();
+                delete P;
+                return P3_ERR_CUDA;
+            }
     const size_t nvals = T.vals.size();
     const size_t bytes = nvals * P->csize;
     if (bytes) {
@@ -1222,7 +1233,7 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
                     }
                     if (i + 1 < a.npass) rs += "x";
                 }
-            } else if (a.kern != p3::KIND_GENERIC) {
+            } else if (a.kern != p3::KIND_GENERIC && a.kern != p3::KIND_LINE32) {
                 // power-of-two kernels: radix E = nfft / tpl while it divides, then the rest
                 const int E = a.nfft / a.tpl;
                 int n = a.nfft;

@@ -830,7 +830,13 @@ template <typename T> __host__ __device__ constexpr int col_E(int N, int mode)
 }
 template <typename T> __host__ __device__ constexpr int col_B(int N)
 {
-    return sizeof(T) == 4 ? (N <= 64 ? 64 : N <= 128 ? 32 : N <= 256 ? 16 : N <= 2048 ? 8 : 4)
+#ifndef P3_B512
+#define P3_B512 8
+#endif
+#ifndef P3_B256
+#define P3_B256 16
+#endif
+    return sizeof(T) == 4 ? (N <= 64 ? 64 : N <= 128 ? 32 : N <= 256 ? P3_B256 : N <= 512 ? P3_B512 : N <= 2048 ? 8 : 4)
                           : (N <= 64 ? 64 : N <= 128 ? 32 : N <= 256 ? 16 : N <= 512 ? 8 : N <= 2048 ? 4 : 2);
 }
 
