@@ -116,7 +116,7 @@ cudaError_t fix64_launch(const StageArgs& a0, cudaStream_t st)
     line_magic(a.out, nl);
     generic_consts(a);
     void* args[] = {&a};
-    return cudaLaunchKernel(pick(a.fix >> 5, a.fix & 31), dim3((unsigned)grid), dim3((unsigned)a.threads), args, a.smem, st);
+    return launch_overlapped(pick(a.fix >> 5, a.fix & 31), (unsigned)grid, (unsigned)a.threads, args, a.smem, st);
 }
 
 }  // namespace p3

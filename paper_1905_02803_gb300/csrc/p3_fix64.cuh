@@ -38,6 +38,7 @@
 #include <cuda_runtime.h>
 
 #include "p3_internal.h"
+#include "p3_launch.cuh"
 
 // the arithmetic below also builds for the host, where the tests pin it
 #define P3_FX_HD __host__ __device__ __forceinline__
@@ -704,6 +705,7 @@ __device__ __forceinline__ void pass(const StageArgs& a, Q* s, Shared& sh, Threa
     }
 
     // positions (j / Ns) Ns R + j mod Ns + r Ns
+    if (last) stage_ending();
     if constexpr (!out_staged<K>()) {
         if (last) {
             const LineExp le = line_exp(th.sexp, th.bad);
@@ -873,6 +875,7 @@ __global__ void __launch_bounds__(kThreads, CAP <= 10 ? 4 : 2) kernel(const __gr
         sh.bout2[tid] = bo2;
     }
     __syncthreads();
+    stage_begin();
 
     if constexpr (in_staged<K>()) {
         if constexpr (K == K_RP) {

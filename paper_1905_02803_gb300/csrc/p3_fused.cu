@@ -454,8 +454,6 @@ bool fused_configure(PlaneArgs& f, const StageArgs& x, const StageArgs& y, int d
     return true;
 }
 
-cudaError_t fused_prepare() { return cudaSuccess; }
-
 cudaError_t fused_launch(const PlaneArgs& f, cudaStream_t s)
 {
     void* fn = pick(f.kx, f.ky, f.dir, f.tp != 0);

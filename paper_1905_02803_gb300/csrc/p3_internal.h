@@ -7,6 +7,9 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#ifndef P3_PDL
+#define P3_PDL 1
+#endif
 namespace p3 {
 
 // Largest radix sequence a line plan can hold (mixed 2/3/5/7 factorizations
@@ -176,13 +179,30 @@ inline void generic_consts(StageArgs& a)
     if (a.blue) pass_consts(a.mpc, a.m, a.mpass, a.mrad, a.tpl, 1);
 }
 
+// Launches a stage kernel that starts with stage_begin() (p3_launch.cuh): its
+// blocks may be resident, up to that point, while the stage before it in the
+// stream finishes.
+inline cudaError_t launch_overlapped(void* fn, unsigned grid, unsigned block, void** args, size_t smem, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = P3_PDL;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
 // Launch one stage (defined in p3_kernels.cu).  Returns the launch error.
 cudaError_t launch_stage_f32(const StageArgs& a, cudaStream_t s);
 cudaError_t launch_stage_f64(const StageArgs& a, cudaStream_t s);
-// One-time kernel attribute set-up for the current device (max dynamic smem):
-// of the kernels that any plan may take, and of a configured stage's own.
-cudaError_t prepare_kernels();
-cudaError_t prepare_stage(const StageArgs& a);
+// Attribute set-up (max dynamic shared memory) of the kernel that a configured
+// stage takes, for the current device.
+cudaError_t prepare_stage(const StageArgs& a, bool f32);
 
 // FP64 fixed-point kernels (p3_fix64.cu).  a.tw and a.tw2 hold twiddles in
 // fixed point there: {re high, re low, im high, im low} of exp(-2 pi i k / n)
@@ -218,7 +238,7 @@ cudaError_t line32_launch(const StageArgs& a, cudaStream_t s);
 bool pow2_configure(StageArgs& a, size_t csize, bool allow_tma);
 // Encodes a.tmap for a stage with a.tma set, from a.src (p3_pow2.cu).
 cudaError_t pow2_encode_tma(StageArgs& a);
-cudaError_t pow2_prepare();
+cudaError_t pow2_prepare(const StageArgs& a, bool f32);
 cudaError_t pow2_launch(const StageArgs& a, bool f32, cudaStream_t s);
 
 // Fused X + Y stages over z-planes (p3_fused.cu).  One persistent launch
@@ -254,7 +274,6 @@ struct PlaneArgs {
 // Returns true when a plane-fused kernel exists for these X and Y stages;
 // fills f (except buffers and counters).
 bool fused_configure(PlaneArgs& f, const StageArgs& x, const StageArgs& y, int dir, size_t csize, bool tp);
-cudaError_t fused_prepare();
 cudaError_t fused_launch(const PlaneArgs& f, cudaStream_t s);
 
 

@@ -18,6 +18,7 @@
 
 #include "p3_dft.cuh"
 #include "p3_internal.h"
+#include "p3_launch.cuh"
 
 namespace p3 {
 namespace {
@@ -701,6 +702,7 @@ __global__ void __launch_bounds__(kGenThreads, (sizeof(T) == 4 ? P3_GEN_MINB : P
     stage_kernel(const __grid_constant__ StageArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    stage_begin();
     stage_tile<T>(a, blockIdx.x, smem_raw);
 }
 
@@ -715,8 +717,8 @@ cudaError_t launch_stage(const StageArgs& a0, cudaStream_t st)
     line_magic(a.in, nl);
     line_magic(a.out, nl);
     generic_consts(a);
-    stage_kernel<T><<<(unsigned)grid, a.threads, a.smem, st>>>(a);
-    return cudaGetLastError();
+    void* args[] = {&a};
+    return launch_overlapped((void*)stage_kernel<T>, (unsigned)grid, (unsigned)a.threads, args, a.smem, st);
 }
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p)
@@ -847,21 +849,17 @@ cudaError_t launch_stage_f64(const StageArgs& a, cudaStream_t s)
     return a.kern != KIND_GENERIC ? pow2_launch(a, false, s) : launch_stage<double>(a, s);
 }
 
-cudaError_t prepare_stage(const StageArgs& a)
+cudaError_t prepare_stage(const StageArgs& a, bool f32)
 {
-    return a.kern == KIND_FIX64 ? fix64_prepare(a) : a.kern == KIND_LINE32 ? line32_prepare(a) : cudaSuccess;
-}
-
-cudaError_t prepare_kernels()
-{
-    cudaError_t e = cudaFuncSetAttribute(stage_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         227 * 1024);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(stage_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    if (e != cudaSuccess) return e;
-    e = pow2_prepare();
-    if (e != cudaSuccess) return e;
-    return tc_prepare();
+    if (a.tc) return tc_prepare();
+    switch (a.kern) {
+    case KIND_FIX64: return fix64_prepare(a);
+    case KIND_LINE32: return line32_prepare(a);
+    case KIND_GENERIC:
+        return cudaFuncSetAttribute(f32 ? (const void*)stage_kernel<float> : (const void*)stage_kernel<double>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    default: return pow2_prepare(a, f32);
+    }
 }
 
 }  // namespace p3

@@ -23,6 +23,7 @@
 
 #include "p3_dft.cuh"
 #include "p3_internal.h"
+#include "p3_launch.cuh"
 
 namespace p3 {
 namespace l32 {
@@ -183,6 +184,7 @@ __device__ __forceinline__ void pass(const StageArgs& a, C* s, const Shared& sh,
 #pragma unroll
     for (int b = 0; b < BM; ++b) Dft<C, float, R>::run(v + b * R);
 
+    if (last) stage_ending();
     if constexpr (!out_staged<K>()) {
         if (last) {
             const ll es = a.out.es;
@@ -296,6 +298,7 @@ template <int K> __global__ void __launch_bounds__(kThreads, P3_L32_MINB) kernel
         sh.bout[tid] = base_of(a.out, L);
     }
     __syncthreads();
+    stage_begin();
 
     if constexpr (in_staged<K>()) {
         const C* F = static_cast<const C*>(a.src);
@@ -447,6 +450,7 @@ __device__ __forceinline__ void row_pass(const StageArgs& a, C* s, const Row& th
 #pragma unroll
     for (int b = 0; b < BM; ++b) Dft<C, float, R>::run(v + b * R);
 
+    if (last) stage_ending();
     const bool direct = last && (K == K_C2R || K == K_CP);
     if (!direct) __syncthreads();  // every thread has read its inputs
     int qq = q0, rr = r0;
@@ -524,6 +528,7 @@ template <int K> __global__ void __launch_bounds__(kThreads, P3_L32_ROW_MINB) ro
     }
     const int ps = a.LDB;
     C* sl = s + l * rpitch(n, ps);
+    stage_begin();
     row_any<K, true>(a, sl, th, 0, 1);
     int Ns = a.rad[0];
     for (int p = 1; p < a.npass; ++p) {

@@ -1055,18 +1055,14 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
         delete P;
         return P3_ERR_CUDA;
     }
-    if (p3::prepare_kernels() != cudaSuccess) {
-        cudaGetLastError();
-        delete P;
-        return P3_ERR_CUDA;
-    }
     for (int d = 0; d < 3; ++d)
-        for (const Stage& s : P->st[d])
-            if (p3::prepare_stage(s.a) != cudaSuccess) {
-                cudaGetLastError();
-                delete P;
-                return P3_ERR_CUDA;
-            }
+        for (const auto* list : {&P->st[d], &unfused[d]})
+            for (const Stage& s : *list)
+                if (p3::prepare_stage(s.a, prec == P3_F32) != cudaSuccess) {
+                    cudaGetLastError();
+                    delete P;
+                    return P3_ERR_CUDA;
+                }
     const size_t nvals = T.vals.size();
     const size_t bytes = nvals * P->csize;
     if (bytes) {

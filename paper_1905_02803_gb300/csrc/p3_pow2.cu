@@ -83,41 +83,26 @@ static bool configure(StageArgs& a, size_t csize, bool allow_tma)
     return true;
 }
 
-cudaError_t pow2_prepare()
+// The kernel of a configured stage.
+static void* kernel_of(const StageArgs& a, bool f32)
 {
-    for (int f = 0; f < 2; ++f)
-        for (int kind = KIND_COL_DD; kind <= KIND_ROW_C2R; ++kind)
-            for (int N = 64; N <= 4096; N *= 2)
-                for (int inv = 0; inv < 2; ++inv)
-                    for (int sym = 0; sym < 3; ++sym) {
-                            void* fn = f == 0 ? pow2_pick_f32(kind, N, inv, sym) : pow2_pick_f64(kind, N, inv, sym);
-                            if (f == 0 && kind == KIND_COL_SD && inv && sym == 0) {
-                                void* fb = pow2_pick_zbulk_f32(N);
-                                if (fb && cudaFuncSetAttribute(fb, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                               227 * 1024) != cudaSuccess)
-                                    return cudaGetLastError();
-                            }
-                            if (f == 0 && kind == KIND_COL_DS && !inv) {
-                                void* ft = pow2_pick_tma_f32(N, sym);
-                                if (ft && cudaFuncSetAttribute(ft, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                               227 * 1024) != cudaSuccess)
-                                    return cudaGetLastError();
-                            }
-                            if (!fn) continue;
-                            cudaError_t e =
-                                cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-                            if (e != cudaSuccess) return e;
-                        }
-    return cudaSuccess;
+    const bool inv = a.sign > 0;
+    const int sym = sym_of(a);
+    return a.tma == 2 ? pow2_pick_zbulk_f32(a.nfft)
+           : a.tma    ? pow2_pick_tma_f32(a.nfft, sym)
+                      : (f32 ? pow2_pick_f32(a.kern, a.nfft, inv, sym) : pow2_pick_f64(a.kern, a.nfft, inv, sym));
+}
+
+cudaError_t pow2_prepare(const StageArgs& a, bool f32)
+{
+    void* fn = kernel_of(a, f32);
+    if (!fn) return cudaErrorInvalidDeviceFunction;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
 }
 
 cudaError_t pow2_launch(const StageArgs& a, bool f32, cudaStream_t st)
 {
-    const bool inv = a.sign > 0;
-    const int sym = sym_of(a);
-    void* fn = a.tma == 2 ? pow2_pick_zbulk_f32(a.nfft)
-               : a.tma ? pow2_pick_tma_f32(a.nfft, sym)
-                     : (f32 ? pow2_pick_f32(a.kern, a.nfft, inv, sym) : pow2_pick_f64(a.kern, a.nfft, inv, sym));
+    void* fn = kernel_of(a, f32);
     if (!fn) return cudaErrorInvalidDeviceFunction;
     if (a.nlines <= 0) return cudaSuccess;
     long long grid = (a.nlines + a.B - 1) / a.B;
@@ -126,7 +111,7 @@ cudaError_t pow2_launch(const StageArgs& a, bool f32, cudaStream_t st)
     line_magic(m.in, m.nlines);
     line_magic(m.out, m.nlines);
     void* args[] = {&m};
-    return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(m.threads), args, m.smem, st);
+    return launch_overlapped(fn, (unsigned)grid, (unsigned)m.threads, args, m.smem, st);
 }
 
 // cuTensorMapEncodeTiled, from the driver through the runtime (resolved once)

@@ -31,6 +31,7 @@
 
 #include "p3_dft.cuh"
 #include "p3_internal.h"
+#include "p3_launch.cuh"
 
 namespace p3 {
 namespace pw {
@@ -239,7 +240,9 @@ template <> struct Vec4<float> { typedef float4 t; };
 // x[e - 1] below M and -x[N - 1 - e] above; output k is i times bin k + 1).
 // One tile of B lines (tile index `tile`, lines offset by `off` elements in
 // both arrays); s: the tile's shared memory.
-template <typename T, int N, int E, int B, int MODE, bool INV, int SYM, int LP = LD_DEF, int SP = ST_DEF>
+// STAGE: the tile is all that its block does of a stage (stage_ending).
+template <typename T, int N, int E, int B, int MODE, bool INV, int SYM, int LP = LD_DEF, int SP = ST_DEF,
+          bool STAGE = false>
 __device__ __forceinline__ void col_tile(const StageArgs& a, long long tile, long long off,
                                          typename CxT<T>::t* s)
 {
@@ -315,6 +318,7 @@ __device__ __forceinline__ void col_tile(const StageArgs& a, long long tile, lon
     }
     pass_compute<C, T, N, E, 0>(v, t, tw, 1);
     ColRest<C, T, N, E, B, SWZ, 1, NP>::run(v, s, l, t, tw);
+    if constexpr (STAGE) stage_ending();
 
     typedef PassIdx<N, E, NP - 1> PLast;
     if constexpr (MODE != 1) {
@@ -381,7 +385,8 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
     col_kernel(const __grid_constant__ StageArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    col_tile<T, N, E, B, MODE, INV, SYM>(a, blockIdx.x, 0, reinterpret_cast<typename CxT<T>::t*>(smem_raw));
+    stage_begin();
+    col_tile<T, N, E, B, MODE, INV, SYM, LD_DEF, ST_DEF, true>(a, blockIdx.x, 0, reinterpret_cast<typename CxT<T>::t*>(smem_raw));
 }
 
 // ---------------------------------------------------------------------------
@@ -474,6 +479,7 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
     const long long L0 = (long long)blockIdx.x * B;
     if (tid == 0) copy_bar_init(bar, a.wait_extra);
     __syncthreads();
+    stage_begin();
     if (tid == 0) {
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(TX) : "memory");
 #pragma unroll
@@ -505,6 +511,7 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
         }
     pass_compute<C, T, N, E, 0>(v, t, tw, 1);
     ColRest<C, T, N, E, B, true, 1, NP>::run(v, s, l, t, tw);  // starts with a block barrier
+    stage_ending();
 
     typedef PassIdx<N, E, NP - 1> PLast;
     __syncthreads();
@@ -602,7 +609,7 @@ template <class C, class T, int N, int E, int NP, int TS> struct RowRest<C, T, N
 
 // Rows L0 .. L0 + B - 1 (those below Lend) of a row stage; s: the tile's
 // shared memory.
-template <typename T, int N, int E, int B, int OPR, int LP = LD_DEF, int SP = ST_DEF>
+template <typename T, int N, int E, int B, int OPR, int LP = LD_DEF, int SP = ST_DEF, bool STAGE = false>
 __device__ __forceinline__ void row_tile(const StageArgs& a, long long L0, long long Lend, typename CxT<T>::t* s)
 {
     typedef typename CxT<T>::t C;
@@ -648,6 +655,7 @@ __device__ __forceinline__ void row_tile(const StageArgs& a, long long L0, long 
     }
     pass_compute<C, T, N, E, 0>(v, t, tw2, 2);
     RowRest<C, T, N, E, 1, NP, 0>::run(v, srow, t, static_cast<const C*>(a.twr));
+    if constexpr (STAGE) stage_ending();
 
     if constexpr (OPR == 0) {
         row_sync<N / E>();
@@ -686,8 +694,9 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
     row_kernel(const __grid_constant__ StageArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    row_tile<T, N, E, B, OPR>(a, (long long)blockIdx.x * B, a.nlines,
-                              reinterpret_cast<typename CxT<T>::t*>(smem_raw));
+    stage_begin();
+    row_tile<T, N, E, B, OPR, LD_DEF, ST_DEF, true>(a, (long long)blockIdx.x * B, a.nlines,
+                                                    reinterpret_cast<typename CxT<T>::t*>(smem_raw));
 }
 
 // ---------------------------------------------------------------------------
@@ -738,6 +747,7 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
     C v[E];
     typedef PassIdx<N, E, 0> P0;
     typedef PassIdx<N, E, NP - 1> PLast;
+    stage_begin();
     if constexpr (BULK) {
         const unsigned bar = smem_u32(base + zrow_area<T, N, E, B>());
         const long long left = a.nlines - L0;
@@ -779,6 +789,7 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
     }
     pass_compute<C, T, N, E, 0>(v, t, tw, 1);
     RowRest<C, T, N, E, 1, NP, 0>::run(v, s + l * S::RP, t, static_cast<const C*>(a.twr));
+    stage_ending();
     __syncthreads();  // the result tile overlaps other lines' exchange rows
     {
         const int u = PLast::out_u(t);
@@ -830,13 +841,7 @@ template <typename T> __host__ __device__ constexpr int col_E(int N, int mode)
 }
 template <typename T> __host__ __device__ constexpr int col_B(int N)
 {
-#ifndef P3_B512
-#define P3_B512 8
-#endif
-#ifndef P3_B256
-#define P3_B256 16
-#endif
-    return sizeof(T) == 4 ? (N <= 64 ? 64 : N <= 128 ? 32 : N <= 256 ? P3_B256 : N <= 512 ? P3_B512 : N <= 2048 ? 8 : 4)
+    return sizeof(T) == 4 ? (N <= 64 ? 64 : N <= 128 ? 32 : N <= 256 ? 16 : N <= 2048 ? 8 : 4)
                           : (N <= 64 ? 64 : N <= 128 ? 32 : N <= 256 ? 16 : N <= 512 ? 8 : N <= 2048 ? 4 : 2);
 }
 
