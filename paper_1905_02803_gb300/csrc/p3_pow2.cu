@@ -7,15 +7,21 @@
 
 namespace p3 {
 
-void* pow2_pick_f32(int kind, int N, bool inv, int sym);
+void* pow2_pick_f32(int kind, int N, bool inv, int sym, bool wide);
 void* pow2_pick_f64(int kind, int N, bool inv, int sym);
-void pow2_shape_f32(int kind, int N, int* B, int* tpl, size_t* smem);
+void pow2_shape_f32(int kind, int N, bool wide, int* B, int* tpl, size_t* smem);
 void pow2_shape_f64(int kind, int N, int* B, int* tpl, size_t* smem);
 
-void* pow2_pick_tma_f32(int N, int sym);
-size_t pow2_tma_smem_f32(int N, int sym);
+void* pow2_pick_tma_f32(int N, int sym, bool wide);
+size_t pow2_tma_smem_f32(int N, int sym, bool wide);
 void* pow2_pick_zbulk_f32(int N);
 size_t pow2_zbulk_smem_f32(int N);
+
+// Whether a column stage takes the 16-line tiles (see kWideB in p3_pow2.cuh).
+static bool wide_of(int kind, int N, long long es)
+{
+    return N == 512 && (kind == KIND_COL_DD || kind == KIND_COL_DS) && es >= 65536 / 8;
+}
 
 // Column-kernel symmetry variant of a stage: 0 plain, 1 DCT-I, 2 DST-I.
 static int sym_of(const StageArgs& a) { return a.op == OP_DCT1 ? 1 : a.op == OP_DST1 ? 2 : 0; }
@@ -56,7 +62,8 @@ static bool configure(StageArgs& a, size_t csize, bool allow_tma)
     }
     int B = 1, tpl = 1;
     size_t smem = 0;
-    if (f32) pow2_shape_f32(kind, N, &B, &tpl, &smem);
+    const bool wide = f32 && wide_of(kind, N, a.in.es);
+    if (f32) pow2_shape_f32(kind, N, wide, &B, &tpl, &smem);
     else pow2_shape_f64(kind, N, &B, &tpl, &smem);
     a.B = B;
     a.LDB = B;
@@ -71,7 +78,7 @@ static bool configure(StageArgs& a, size_t csize, bool allow_tma)
     if (f32 && allow_tma && kind == KIND_COL_DS && N >= 256 && N <= 2048 && a.in.lstride == 1 &&
         a.in.per >= a.nlines && a.in.es % 2 == 0 && a.in.es >= a.nlines && (B % 2) == 0) {
         a.tma = 1;
-        a.smem = pow2_tma_smem_f32(N, sym_of(a));
+        a.smem = pow2_tma_smem_f32(N, sym_of(a), wide);
     }
     // bulk-copied tile for the row-style ZYX load: plain FFT lines that lie
     // one after another in memory
@@ -88,9 +95,10 @@ static void* kernel_of(const StageArgs& a, bool f32)
 {
     const bool inv = a.sign > 0;
     const int sym = sym_of(a);
+    const bool wide = f32 && wide_of(a.kern, a.nfft, a.in.es);
     return a.tma == 2 ? pow2_pick_zbulk_f32(a.nfft)
-           : a.tma    ? pow2_pick_tma_f32(a.nfft, sym)
-                      : (f32 ? pow2_pick_f32(a.kern, a.nfft, inv, sym) : pow2_pick_f64(a.kern, a.nfft, inv, sym));
+           : a.tma    ? pow2_pick_tma_f32(a.nfft, sym, wide)
+                      : (f32 ? pow2_pick_f32(a.kern, a.nfft, inv, sym, wide) : pow2_pick_f64(a.kern, a.nfft, inv, sym));
 }
 
 cudaError_t pow2_prepare(const StageArgs& a, bool f32)

@@ -845,6 +845,16 @@ template <typename T> __host__ __device__ constexpr int col_B(int N)
                           : (N <= 64 ? 64 : N <= 128 ? 32 : N <= 256 ? 16 : N <= 512 ? 8 : N <= 2048 ? 4 : 2);
 }
 
+// FP32 column stages of 512 points whose elements lie far apart (the Z stages
+// of large planes) take 16 lines per tile instead of 8: 128-byte runs.
+// Measured at 512^3: Z in place 274 / 295 -> 227 / 218 us, ZYX store 195 -> 180
+// us; Y lines, whose neighbouring tiles share a DRAM page, lose (219 -> 229
+// us) and keep 8.  The line lies at 64 KB between elements (Y: at most 32 KB
+// for rows of up to 4096 bins; Z of a 512-point plane 1 MB).
+constexpr int kWideB = 16;
+constexpr long long kWideStride = 65536 / 8;  // complex elements
+__host__ __device__ constexpr bool has_wide(int N) { return N == 512; }
+
 // Row-style ZYX-load kernel for FP32 lines of 256 .. 2048 points (a line's
 // threads fit in one warp up to 1024 points; two warps at 2048).
 #ifndef P3_ZROW

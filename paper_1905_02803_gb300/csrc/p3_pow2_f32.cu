@@ -6,8 +6,10 @@ namespace p3 {
 namespace {
 using namespace pw;
 
-template <int N, int MODE, bool INV, int SYM> void* col_fn()
+template <int N, int MODE, bool INV, int SYM> void* col_fn(bool wide)
 {
+    if constexpr (has_wide(N) && MODE != 2)
+        if (wide) return (void*)col_kernel<float, N, col_E<float>(N, MODE), kWideB, MODE, INV, SYM>;
     return (void*)col_kernel<float, N, col_E<float>(N, MODE), col_B<float>(N), MODE, INV, SYM>;
 }
 template <int N, bool INV, int SYM> void* zrow_fn()
@@ -17,18 +19,20 @@ template <int N, bool INV, int SYM> void* zrow_fn()
     else
         return nullptr;
 }
-template <int N, int SYM> void* tma_fn()
+template <int N, int SYM> void* tma_fn(bool wide)
 {
+    if constexpr (has_wide(N))
+        if (wide) return (void*)col_kernel_tma<float, N, col_E<float>(N, 1), kWideB, SYM>;
     return (void*)col_kernel_tma<float, N, col_E<float>(N, 1), col_B<float>(N), SYM>;
 }
 template <int N, int OPR> void* row_fn() { return (void*)row_kernel<float, N, row_E<float>(N), row_B<float>(N), OPR>; }
 
 // sym: 0 plain, 1 Chebyshev (DCT-I), 2 sine (DST-I, forward sign only)
 #define P3_COL_PICK(FN, MODE) \
-    (sym == 2 ? (inv ? (void*)nullptr : FN<N, MODE, false, 2>()) \
-     : inv ? (sym ? FN<N, MODE, true, 1>() : FN<N, MODE, true, 0>()) \
-           : (sym ? FN<N, MODE, false, 1>() : FN<N, MODE, false, 0>()))
-template <int N> void* pick_n(int kind, bool inv, int sym)
+    (sym == 2 ? (inv ? (void*)nullptr : FN<N, MODE, false, 2>(wide)) \
+     : inv ? (sym ? FN<N, MODE, true, 1>(wide) : FN<N, MODE, true, 0>(wide)) \
+           : (sym ? FN<N, MODE, false, 1>(wide) : FN<N, MODE, false, 0>(wide)))
+template <int N> void* pick_n(int kind, bool inv, int sym, bool wide)
 {
     switch (kind) {
     case KIND_COL_DD: return P3_COL_PICK(col_fn, 0);
@@ -47,16 +51,16 @@ template <int N> void* pick_n(int kind, bool inv, int sym)
 #undef P3_COL_PICK
 }  // namespace
 
-void* pow2_pick_f32(int kind, int N, bool inv, int sym)
+void* pow2_pick_f32(int kind, int N, bool inv, int sym, bool wide)
 {
     switch (N) {
-    case 64: return pick_n<64>(kind, inv, sym);
-    case 128: return pick_n<128>(kind, inv, sym);
-    case 256: return pick_n<256>(kind, inv, sym);
-    case 512: return pick_n<512>(kind, inv, sym);
-    case 1024: return pick_n<1024>(kind, inv, sym);
-    case 2048: return pick_n<2048>(kind, inv, sym);
-    case 4096: return pick_n<4096>(kind, inv, sym);
+    case 64: return pick_n<64>(kind, inv, sym, wide);
+    case 128: return pick_n<128>(kind, inv, sym, wide);
+    case 256: return pick_n<256>(kind, inv, sym, wide);
+    case 512: return pick_n<512>(kind, inv, sym, wide);
+    case 1024: return pick_n<1024>(kind, inv, sym, wide);
+    case 2048: return pick_n<2048>(kind, inv, sym, wide);
+    case 4096: return pick_n<4096>(kind, inv, sym, wide);
     default: return nullptr;
     }
 }
@@ -85,19 +89,20 @@ size_t pow2_zbulk_smem_f32(int N)
 }
 
 // TMA-staged ZYX-store kernels (FP32, 256 .. 2048 points): kernel and dynamic shared memory
-void* pow2_pick_tma_f32(int N, int sym)
+void* pow2_pick_tma_f32(int N, int sym, bool wide)
 {
     switch (N) {
-    case 256: return sym == 2 ? tma_fn<256, 2>() : sym ? tma_fn<256, 1>() : tma_fn<256, 0>();
-    case 512: return sym == 2 ? tma_fn<512, 2>() : sym ? tma_fn<512, 1>() : tma_fn<512, 0>();
-    case 1024: return sym == 2 ? tma_fn<1024, 2>() : sym ? tma_fn<1024, 1>() : tma_fn<1024, 0>();
-    case 2048: return sym == 2 ? tma_fn<2048, 2>() : sym ? tma_fn<2048, 1>() : tma_fn<2048, 0>();
+    case 256: return sym == 2 ? tma_fn<256, 2>(wide) : sym ? tma_fn<256, 1>(wide) : tma_fn<256, 0>(wide);
+    case 512: return sym == 2 ? tma_fn<512, 2>(wide) : sym ? tma_fn<512, 1>(wide) : tma_fn<512, 0>(wide);
+    case 1024: return sym == 2 ? tma_fn<1024, 2>(wide) : sym ? tma_fn<1024, 1>(wide) : tma_fn<1024, 0>(wide);
+    case 2048: return sym == 2 ? tma_fn<2048, 2>(wide) : sym ? tma_fn<2048, 1>(wide) : tma_fn<2048, 0>(wide);
     default: return nullptr;
     }
 }
-size_t pow2_tma_smem_f32(int N, int sym)
+size_t pow2_tma_smem_f32(int N, int sym, bool wide)
 {
     using namespace pw;
+    if (wide && N == 512) return col_tma_smem<float, 512, kWideB>(sym);
     switch (N) {
     case 256: return col_tma_smem<float, 256, col_B<float>(256)>(sym);
     case 512: return col_tma_smem<float, 512, col_B<float>(512)>(sym);
@@ -107,7 +112,7 @@ size_t pow2_tma_smem_f32(int N, int sym)
     }
 }
 
-void pow2_shape_f32(int kind, int N, int* B, int* tpl, size_t* smem)
+void pow2_shape_f32(int kind, int N, bool wide, int* B, int* tpl, size_t* smem)
 {
     using namespace pw;
     if (kind == KIND_ROW_R2C || kind == KIND_ROW_C2R) {
@@ -127,7 +132,7 @@ void pow2_shape_f32(int kind, int N, int* B, int* tpl, size_t* smem)
         }
     } else {
         const int mode = kind == KIND_COL_SD ? 2 : kind == KIND_COL_DS ? 1 : 0;
-        *B = col_B<float>(N);
+        *B = wide && has_wide(N) && mode != 2 ? kWideB : col_B<float>(N);
         const size_t slots = (size_t)(cpad_c(N - 1) + 1) * (size_t)(*B);
         *tpl = N / col_E<float>(N, mode);
         *smem = slots * sizeof(float) * 2;
