@@ -526,7 +526,7 @@ const char* kern_name(const StageArgs& a)
     }
     if (a.tc) return "tc_split_col";
     if (tma == 2) return "pow2_zrow_bulk";
-    if (tma) return "pow2_col_zyx_store_tma";
+    if (tma) return k == p3::KIND_COL_DS ? "pow2_col_zyx_store_tma" : "pow2_col_tma";
     switch (k) {
     case p3::KIND_COL_DD: return "pow2_col";
     case p3::KIND_COL_DS: return "pow2_col_zyx_store";

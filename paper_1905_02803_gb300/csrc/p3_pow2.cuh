@@ -318,7 +318,9 @@ __device__ __forceinline__ void col_tile(const StageArgs& a, long long tile, lon
     }
     pass_compute<C, T, N, E, 0>(v, t, tw, 1);
     ColRest<C, T, N, E, B, SWZ, 1, NP>::run(v, s, l, t, tw);
-    if constexpr (STAGE) stage_ending();
+    // (in the 8-line strided kernels of 512 points and more the early call costs
+    // more than it hides: Y of 512^3 220 us with it, 214 without)
+    if constexpr (STAGE && (MODE != 0 || N < 512 || B >= 16)) stage_ending();
 
     typedef PassIdx<N, E, NP - 1> PLast;
     if constexpr (MODE != 1) {
@@ -390,7 +392,8 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
 }
 
 // ---------------------------------------------------------------------------
-// ZYX-store column kernel with a TMA-staged input tile (forward Z stage).
+// Column kernel with a TMA-staged input tile (Z stages: ZYX store, or with
+// ZYX = false the strided store of the XYZ layout in either direction).
 // The tile's B lines are adjacent in memory and their elements es apart, so
 // the tile is a 2D box of the array (lines inner, elements outer): one thread
 // arms an mbarrier with the tile's byte count and issues the tensor copies
@@ -454,11 +457,12 @@ template <typename T, int N, int B, int SYM> __host__ __device__ constexpr size_
     return (size_t)((tma_rows<N, SYM>() + kTmaRows - 1) / kTmaRows) * kTmaRows * B * 2 * sizeof(T);
 }
 
-template <typename T, int N, int E, int B, int SYM>
+template <typename T, int N, int E, int B, int SYM, bool ZYX = true, bool INV = false>
 __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeof(T), E>::value))
     col_kernel_tma(const __grid_constant__ StageArgs a)
 {
     static_assert(sizeof(T) == 4, "TMA tiles of 8-byte complex elements");
+    static_assert(!INV || (!ZYX && SYM != 2), "inverse: strided store; the sine transform has the forward sign both ways");
     constexpr bool DCT = SYM == 1, DST = SYM == 2;
     typedef typename CxT<T>::t C;
     typedef P2<N, E> PL;
@@ -507,13 +511,33 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
             } else {
                 x = s[(DCT ? (e <= M ? e : N - e) : e) * B + l];
             }
-            v[b * P0::R + r] = x;
+            v[b * P0::R + r] = INV ? swp(x) : x;
         }
     pass_compute<C, T, N, E, 0>(v, t, tw, 1);
-    ColRest<C, T, N, E, B, true, 1, NP>::run(v, s, l, t, tw);  // starts with a block barrier
-    stage_ending();
+    ColRest<C, T, N, E, B, ZYX, 1, NP>::run(v, s, l, t, tw);  // starts with a block barrier
+    if constexpr (N < 1024) stage_ending();  // longer tiles: costs more than it hides (1024^3: 4 us a stage)
 
     typedef PassIdx<N, E, NP - 1> PLast;
+    if constexpr (!ZYX) {
+        if (L0 + l < a.nlines) {
+            C* dst = static_cast<C*>(a.dst) + lbase(a.out, L0 + l);
+            const long long es = a.out.es;
+            const int u = PLast::out_u(t);
+#pragma unroll
+            for (int b = 0; b < PLast::BM; ++b)
+#pragma unroll
+                for (int r = 0; r < PLast::R; ++r) {
+                    const int e = u + PLast::out_K(b, r);
+                    const C x = v[b * PLast::R + r];
+                    if constexpr (DST) {
+                        if (e >= 1 && e < M) dst[(long long)(e - 1) * es] = mk<C>(-x.y, x.x);
+                    } else {
+                        if (!DCT || e <= M) dst[(long long)e * es] = INV ? swp(x) : x;
+                    }
+                }
+        }
+        return;
+    }
     __syncthreads();
     {
         const int u = PLast::out_u(t);
@@ -811,7 +835,7 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
     }
     pass_compute<C, T, N, E, 0>(v, t, tw, 1);
     RowRest<C, T, N, E, 1, NP, 0>::run(v, s + l * S::RP, t, static_cast<const C*>(a.twr));
-    stage_ending();
+    if constexpr (N < 1024) stage_ending();  // longer tiles: costs more than it hides (1024^3: 4 us a stage)
     __syncthreads();  // the result tile overlaps other lines' exchange rows
     {
         const int u = PLast::out_u(t);

@@ -19,11 +19,24 @@ template <int N, bool INV, int SYM> void* zrow_fn()
     else
         return nullptr;
 }
-template <int N, int SYM> void* tma_fn(bool wide)
+template <int N, int B> void* tma_b(int sym, bool zyx, bool inv)
+{
+    constexpr int E = col_E<float>(N, 1);
+    if (zyx)
+        return sym == 2 ? (void*)col_kernel_tma<float, N, E, B, 2>
+               : sym    ? (void*)col_kernel_tma<float, N, E, B, 1>
+                        : (void*)col_kernel_tma<float, N, E, B, 0>;
+    return sym == 2 ? (void*)col_kernel_tma<float, N, E, B, 2, false>
+           : sym    ? (inv ? (void*)col_kernel_tma<float, N, E, B, 1, false, true>
+                          : (void*)col_kernel_tma<float, N, E, B, 1, false>)
+           : inv    ? (void*)col_kernel_tma<float, N, E, B, 0, false, true>
+                    : (void*)col_kernel_tma<float, N, E, B, 0, false>;
+}
+template <int N> void* tma_fn(int sym, bool wide, bool zyx, bool inv)
 {
     if constexpr (has_wide(N))
-        if (wide) return (void*)col_kernel_tma<float, N, col_E<float>(N, 1), kWideB, SYM>;
-    return (void*)col_kernel_tma<float, N, col_E<float>(N, 1), col_B<float>(N), SYM>;
+        if (wide) return tma_b<N, kWideB>(sym, zyx, inv);
+    return tma_b<N, col_B<float>(N)>(sym, zyx, inv);
 }
 template <int N, int OPR> void* row_fn() { return (void*)row_kernel<float, N, row_E<float>(N), row_B<float>(N), OPR>; }
 
@@ -88,14 +101,16 @@ size_t pow2_zbulk_smem_f32(int N)
     }
 }
 
-// TMA-staged ZYX-store kernels (FP32, 256 .. 2048 points): kernel and dynamic shared memory
-void* pow2_pick_tma_f32(int N, int sym, bool wide)
+// TMA-staged column kernels (FP32, 256 .. 2048 points): kernel and dynamic shared
+// memory.  zyx: ZYX store, otherwise the strided store (inv: inverse sign, by
+// swapped parts for Chebyshev lines too, as the kernels with plain loads)
+void* pow2_pick_tma_f32(int N, int sym, bool wide, bool zyx, bool inv)
 {
     switch (N) {
-    case 256: return sym == 2 ? tma_fn<256, 2>(wide) : sym ? tma_fn<256, 1>(wide) : tma_fn<256, 0>(wide);
-    case 512: return sym == 2 ? tma_fn<512, 2>(wide) : sym ? tma_fn<512, 1>(wide) : tma_fn<512, 0>(wide);
-    case 1024: return sym == 2 ? tma_fn<1024, 2>(wide) : sym ? tma_fn<1024, 1>(wide) : tma_fn<1024, 0>(wide);
-    case 2048: return sym == 2 ? tma_fn<2048, 2>(wide) : sym ? tma_fn<2048, 1>(wide) : tma_fn<2048, 0>(wide);
+    case 256: return tma_fn<256>(sym, wide, zyx, inv);
+    case 512: return tma_fn<512>(sym, wide, zyx, inv);
+    case 1024: return tma_fn<1024>(sym, wide, zyx, inv);
+    case 2048: return tma_fn<2048>(sym, wide, zyx, inv);
     default: return nullptr;
     }
 }
