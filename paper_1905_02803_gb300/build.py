@@ -19,7 +19,7 @@ SOURCES = ["p3_plan.cu", "p3_kernels.cu", "p3_pow2.cu", "p3_pow2_f32.cu", "p3_po
            "p3_fix64_ecc.cu", "p3_fix64_ecs.cu", "p3_fix64_row.cu", "p3_fix64_pair.cu", "p3_line32.cu",
            "p3_line32_a.cu", "p3_line32_b.cu"]
 HEADERS = [os.path.join(CSRC, "p3_internal.h"), os.path.join(CSRC, "p3_dft.cuh"), os.path.join(CSRC, "p3_pow2.cuh"),
-           os.path.join(CSRC, "p3_fix64.cuh"), os.path.join(CSRC, "p3_line32.cuh"), os.path.join(CSRC, "p3_launch.cuh"), os.path.join(ROOT, "include", "p3dfft_gb300.h")]
+           os.path.join(CSRC, "p3_fix64.cuh"), os.path.join(CSRC, "p3_line32.cuh"), os.path.join(CSRC, "p3_launch.cuh"), os.path.join(CSRC, "p3_copy.cuh"), os.path.join(ROOT, "include", "p3dfft_gb300.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include")]
 

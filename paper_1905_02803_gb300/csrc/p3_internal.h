@@ -143,9 +143,10 @@ struct StageArgs {
     int fix;           // KIND_FIX64: which of its kernels (32 fx::Kind + largest radix); KIND_LINE32: l32::Kind
     // 1: tensor-core split-precision kernel (p3_tc.cu)
     int tc;
-    // 1: TMA-staged ZYX-store column kernel (input tile by tensor copies);
-    // 2: row-style ZYX-load kernel with a bulk-copied input tile
+    // 1: input tile by tensor copies (tmap); 2: by bulk copies
     int tma;
+    // KIND_LINE32 with bulk copies: slots between the input lines
+    int box;
     // status word of the plan: a bounded device wait that gave up ORs a bit in
     unsigned* err;
     // polls before a wait for a tensor / bulk copy gives up
@@ -229,7 +230,7 @@ constexpr double kFix64MaxPoints = 12582912.0;
 // FP32 line kernels of smooth lengths (p3_line32.cu): configure a stage whose
 // radices are set (false when none applies; shrink halves the lines per CTA
 // that many times), set them up, launch one stage.
-bool line32_configure(StageArgs& a, int shrink);
+bool line32_configure(StageArgs& a, int shrink, bool allow_tma);
 cudaError_t line32_prepare(const StageArgs& a);
 cudaError_t line32_launch(const StageArgs& a, cudaStream_t s);
 

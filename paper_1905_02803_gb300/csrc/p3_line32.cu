@@ -5,16 +5,16 @@
 namespace p3 {
 
 namespace l32 {
-void* fn_a(int k);
+void* fn_a(int k, int tma);
 void* fn_b(int k);
 }  // namespace l32
 
 namespace {
 
-void* pick(int k)
+void* pick(const StageArgs& a)
 {
-    void* f = l32::fn_a(k);
-    return f ? f : l32::fn_b(k);
+    void* f = l32::fn_a(a.fix, a.tma);
+    return f ? f : l32::fn_b(a.fix);
 }
 
 int butterflies(int R)
@@ -70,7 +70,7 @@ int row_pad(int n, int npass, const int* rad, int tpl, int B)
 
 }  // namespace
 
-bool line32_configure(StageArgs& a, int shrink)
+bool line32_configure(StageArgs& a, int shrink, bool allow_tma)
 {
     if (a.blue || a.op == OP_COPY || a.npass < 1 || a.nfft < 2) return false;
     const bool si = a.in_elem_fast, so = a.out_elem_fast;
@@ -96,10 +96,10 @@ bool line32_configure(StageArgs& a, int shrink)
         if (R > 16 || R == 11 || R == 13) return false;
         tpl = tpl > (nb + bm - 1) / bm ? tpl : (nb + bm - 1) / bm;
     }
-    if (tpl > l32::kThreads) return false;
+    if (tpl > l32::kThreadsMost) return false;
     if (k >= l32::K_R2C) {
         // rows: any number of lines per CTA
-        int B = l32::kThreads / tpl;
+        int B = tpl < l32::kThreads ? l32::kThreads / tpl : 1;
         const int ps = row_pad(n, a.npass, a.rad, tpl, B);
         const size_t row = (size_t)l32::rpitch(n, ps) * 8;
         while (B > 1 && B * row > kSmemMost) --B;
@@ -111,8 +111,13 @@ bool line32_configure(StageArgs& a, int shrink)
         a.smem = B * row;
     } else {
         auto pitch = [&](int B) { return l32::staged_kind(k) && B % 2 == 0 ? B + 1 : B; };
+        // up to 8 lines; 16 for the ZYX store, whose odd pitch then has no bank
+        // conflicts (343 points: 117 -> 107 us; the other kinds lose 3 - 15 %)
+        const int wide = k == l32::K_CS || k == l32::K_ECS ? 16 : 8;
         int B = 1;
-        while (2 * B * tpl <= l32::kThreads && 2 * B <= l32::kMaxB && (size_t)n * pitch(2 * B) * 8 <= kSmemMost) B *= 2;
+        while (2 * B * tpl <= (B < wide ? l32::kThreadsMost : l32::kThreads) && 2 * B <= l32::kMaxB &&
+               (size_t)n * pitch(2 * B) * 8 <= kSmemMost)
+            B *= 2;
         // small volumes: narrower tiles while they leave SMs without a CTA
         while (B > 8 && (a.nlines + B - 1) / B < 304) B /= 2;
         B >>= shrink;
@@ -122,18 +127,37 @@ bool line32_configure(StageArgs& a, int shrink)
         a.smem = (size_t)n * a.LDB * 8;
     }
     if (a.smem > kSmemMost) return false;
+    a.tma = 0;
+    a.box = 0;
+    const size_t plain = a.smem;
+    if (allow_tma && k == l32::K_SCI && n % 2 == 0 && a.in.lstride % 2 == 0 && a.in.gstride % 2 == 0 &&
+        a.nlines * n >= (1LL << 22)) {
+        // line copies: lines of whole 16 bytes; the pitch puts a half-warp's
+        // lines on distinct banks.  384^3: 137 -> 121 us, 300 x 324 x 270 80 -> 75;
+        // volumes of a few MB lie in L2, where the barrier costs more than the
+        // loads' latency (24 mixed grids: 1 % slower with it everywhere)
+        a.box = n + 2;
+        while (a.box % 4 != 2) a.box += 2;
+        const size_t tile = (size_t)a.B * a.box * 8;
+        a.smem = ((plain > tile ? plain : tile) + 15) / 16 * 16 + 144;
+        a.tma = 2;
+    }
+    if (a.smem > kSmemMost + 1024) {
+        a.tma = 0;
+        a.box = 0;
+        a.smem = plain;
+    }
     a.tpl = tpl;
     a.threads = (a.B * tpl + 31) / 32 * 32;
     a.kern = KIND_LINE32;
     a.fix = k;
     a.tc = 0;
-    a.tma = 0;
     return true;
 }
 
 cudaError_t line32_prepare(const StageArgs& a)
 {
-    return cudaFuncSetAttribute(pick(a.fix), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMost);
+    return cudaFuncSetAttribute(pick(a), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMost + 1024);
 }
 
 cudaError_t line32_launch(const StageArgs& a0, cudaStream_t st)
@@ -147,7 +171,7 @@ cudaError_t line32_launch(const StageArgs& a0, cudaStream_t st)
     line_magic(a.out, nl);
     generic_consts(a);
     void* args[] = {&a};
-    return launch_overlapped(pick(a.fix), (unsigned)grid, (unsigned)a.threads, args, a.smem, st);
+    return launch_overlapped(pick(a), (unsigned)grid, (unsigned)a.threads, args, a.smem, st);
 }
 
 }  // namespace p3

@@ -21,6 +21,7 @@
 // slower.
 #pragma once
 
+#include "p3_copy.cuh"
 #include "p3_dft.cuh"
 #include "p3_internal.h"
 #include "p3_launch.cuh"
@@ -53,13 +54,8 @@ __host__ __device__ constexpr bool staged_kind(int k) { return k != K_CC && k !=
 template <int K> __host__ __device__ constexpr bool inverse() { return K == K_CCI || K == K_SCI; }
 
 constexpr int kMaxB = 32;
-#ifndef P3_L32_THREADS
-#define P3_L32_THREADS 256
-#endif
-#ifndef P3_L32_MINB
-#define P3_L32_MINB 4
-#endif
-constexpr int kThreads = P3_L32_THREADS;
+constexpr int kThreads = 256;  // threads of a CTA, four CTAs per SM (64 registers) ...
+constexpr int kThreadsMost = 512;  // ... and for long lines, to keep tiles of up to 8 lines
 
 // Butterflies a thread holds per pass (at most 16 values)
 template <int R> __host__ __device__ constexpr int bfly()
@@ -101,7 +97,9 @@ struct Thread {
 // One Stockham pass of radix R over the tile, FIRST from the input (HBM or the
 // staged tile).  Butterfly j reads elements j + r n/R, multiplies by
 // exp(-2 pi i (j mod Ns) r / (Ns R)) and writes (j / Ns) Ns R + j mod Ns + r Ns.
-template <int K, int R, bool FIRST>
+// BULK: the input tile came line by line by bulk copies, element e of line l at
+// l * a.box + e.
+template <int K, bool BULK, int R, bool FIRST>
 __device__ __forceinline__ void pass(const StageArgs& a, C* s, const Shared& sh, const Thread& th, int p, int Ns)
 {
     constexpr int BM = bfly<R>();
@@ -146,20 +144,22 @@ __device__ __forceinline__ void pass(const StageArgs& a, C* s, const Shared& sh,
 #pragma unroll
         for (int b = 0; b < BM; ++b) {
             const int j = clamp(t + b * tpl, nb);
-            const C* sp = s + j * LDB + l;
+            const int es = FIRST && BULK ? 1 : LDB;
+            const C* si = FIRST && BULK ? s + l * a.box : s + l;
+            const C* sp = si + j * es;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 C x = zero;
                 if constexpr (FIRST && extended<K>()) {
                     const int e = j + r * nb, M = n >> 1;
                     if (a.op == OP_DCT1) {
-                        x = s[(e <= M ? e : n - e) * LDB + l];
+                        x = si[(e <= M ? e : n - e) * es];
                     } else if (e != 0 && e != M) {
-                        x = s[(e < M ? e - 1 : n - 1 - e) * LDB + l];
+                        x = si[(e < M ? e - 1 : n - 1 - e) * es];
                         if (e > M) x = mk<C>(-x.x, -x.y);
                     }
                 } else {
-                    x = sp[r * nb * LDB];
+                    x = sp[r * nb * es];
                 }
                 v[b * R + r] = FIRST && inverse<K>() ? swp(x) : x;
             }
@@ -251,12 +251,12 @@ __device__ __forceinline__ void pass(const StageArgs& a, C* s, const Shared& sh,
     __syncthreads();
 }
 
-template <int K, bool FIRST>
+template <int K, bool BULK, bool FIRST>
 __device__ __forceinline__ void pass_any(const StageArgs& a, C* s, const Shared& sh, const Thread& th, int p, int Ns)
 {
     switch (a.rad[p]) {
 #define P3_L32_PASS(R) \
-    case R: pass<K, R, FIRST>(a, s, sh, th, p, Ns); break;
+    case R: pass<K, BULK, R, FIRST>(a, s, sh, th, p, Ns); break;
         P3_L32_PASS(2) P3_L32_PASS(3) P3_L32_PASS(4) P3_L32_PASS(5) P3_L32_PASS(6) P3_L32_PASS(7) P3_L32_PASS(8)
         P3_L32_PASS(9) P3_L32_PASS(10) P3_L32_PASS(12) P3_L32_PASS(14) P3_L32_PASS(15) P3_L32_PASS(16)
 #undef P3_L32_PASS
@@ -283,12 +283,18 @@ template <class F> __device__ __forceinline__ void walk(int rows, int len, F f)
     }
 }
 
-template <int K> __global__ void __launch_bounds__(kThreads, P3_L32_MINB) kernel(const __grid_constant__ StageArgs a)
+template <int K, bool BULK = false>
+__global__ void __launch_bounds__(kThreadsMost, 2) kernel(const __grid_constant__ StageArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Shared sh;
-    C* s = reinterpret_cast<C*>(smem_raw);
+    // a bulk-copied tile is 128-byte aligned (144 bytes more are requested), with
+    // its barrier after it
+    unsigned char* base = BULK ? smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u) : smem_raw;
+    C* s = reinterpret_cast<C*>(base);
     const int tid = threadIdx.x, B = a.B, LDB = a.LDB, n = a.nfft;
+    const unsigned bar = BULK ? smem_u32(base + a.smem - 144) : 0u;
+    if (BULK && tid == 0) copy_bar_init(bar, a.wait_extra);
     const int lb = __ffs(B) - 1;
     const ll L0 = (ll)blockIdx.x * B;
     const int rows = (int)(a.nlines - L0 < B ? a.nlines - L0 : B);
@@ -300,7 +306,14 @@ template <int K> __global__ void __launch_bounds__(kThreads, P3_L32_MINB) kernel
     __syncthreads();
     stage_begin();
 
-    if constexpr (in_staged<K>()) {
+    if constexpr (BULK) {
+        if (tid == 0) {
+            copy_bar_expect(bar, (unsigned)(rows * a.n_in * 8));
+            for (int k = 0; k < rows; ++k)
+                copy_bulk(smem_u32(s + k * a.box), static_cast<const C*>(a.src) + sh.bin[k], (unsigned)(a.n_in * 8), bar);
+        }
+        if (!copy_bar_wait(a, bar)) return;
+    } else if constexpr (in_staged<K>()) {
         const C* F = static_cast<const C*>(a.src);
         walk(rows, a.n_in, [&](int l, int e) { cp_async8(s + e * LDB + l, F + sh.bin[l] + e); });
         asm volatile("cp.async.wait_all;\n" ::: "memory");
@@ -312,10 +325,10 @@ template <int K> __global__ void __launch_bounds__(kThreads, P3_L32_MINB) kernel
     th.t = tid >> lb;
     th.act = th.t < a.tpl;
     th.valid = th.act && th.l < rows;
-    pass_any<K, true>(a, s, sh, th, 0, 1);
+    pass_any<K, BULK, true>(a, s, sh, th, 0, 1);
     int Ns = a.rad[0];
     for (int p = 1; p < a.npass; ++p) {
-        pass_any<K, false>(a, s, sh, th, p, Ns);
+        pass_any<K, BULK, false>(a, s, sh, th, p, Ns);
         Ns *= a.rad[p];
     }
 
@@ -500,10 +513,7 @@ template <int K, bool FIRST> __device__ __forceinline__ void row_any(const Stage
     }
 }
 
-#ifndef P3_L32_ROW_MINB
-#define P3_L32_ROW_MINB 4
-#endif
-template <int K> __global__ void __launch_bounds__(kThreads, P3_L32_ROW_MINB) row_kernel(const __grid_constant__ StageArgs a)
+template <int K> __global__ void __launch_bounds__(kThreadsMost, 2) row_kernel(const __grid_constant__ StageArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* s = reinterpret_cast<C*>(smem_raw);

@@ -494,7 +494,8 @@ void tile_setup(StageArgs& a, size_t csize, unsigned flags, bool fixed)
         return;
     }
     generic_tile_setup(a, csize);
-    if (!p3::pow2_configure(a, csize, !(flags & P3_FLAG_NO_TMA)) && csize == 8) p3::line32_configure(a, 0);
+    if (!p3::pow2_configure(a, csize, !(flags & P3_FLAG_NO_TMA)) && csize == 8)
+        p3::line32_configure(a, 0, !(flags & P3_FLAG_NO_TMA));
     if (flags & P3_FLAG_TC_SPLIT) p3::tc_configure(a, csize);
 }
 
@@ -525,6 +526,7 @@ const char* kern_name(const StageArgs& a)
         return a.out_elem_fast ? "pow2_col_zyx_store_fix64" : a.in_elem_fast ? "pow2_col_zyx_load_fix64" : "pow2_col_fix64";
     }
     if (a.tc) return "tc_split_col";
+    if (k == p3::KIND_LINE32) return tma ? "line32_bulk" : "line32";
     if (tma == 2) return "pow2_zrow_bulk";
     if (tma) return k == p3::KIND_COL_DS ? "pow2_col_zyx_store_tma" : "pow2_col_tma";
     switch (k) {
@@ -533,7 +535,6 @@ const char* kern_name(const StageArgs& a)
     case p3::KIND_COL_SD: return "pow2_col_zyx_load";
     case p3::KIND_ROW_R2C: return "pow2_row_r2c";
     case p3::KIND_ROW_C2R: return "pow2_row_c2r";
-    case p3::KIND_LINE32: return "line32";
     default: return "generic";
     }
 }
@@ -719,7 +720,7 @@ static p3_status tune_generic(p3_plan P, std::string& report)
                     if (a0.kern == p3::KIND_FIX64) {
                         if (!p3::fix64_configure(a, shrink)) break;
                     } else if (a0.kern == p3::KIND_LINE32) {
-                        if (!p3::line32_configure(a, shrink)) break;
+                        if (!p3::line32_configure(a, shrink, a0.tma != 0)) break;
                     } else {
                         generic_tile_setup(a, P->csize);
                         if ((a.B >> shrink) < 1) break;
@@ -735,6 +736,7 @@ static p3_status tune_generic(p3_plan P, std::string& report)
                     a.src = buf[st.src];
                     a.dst = buf[st.dst];
                     a.err = P->derr;
+                    a.spin = P->spin_limit / 2;
                     float ms = 0.f;
                     for (int rep = 0; rep < 4 && rc == P3_OK; ++rep) {
                         if (rep == 1 && cudaEventRecord(e0, sm) != cudaSuccess) rc = P3_ERR_CUDA;

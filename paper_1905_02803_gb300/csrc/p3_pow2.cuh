@@ -31,6 +31,7 @@
 
 #include "p3_dft.cuh"
 #include "p3_internal.h"
+#include "p3_copy.cuh"
 #include "p3_launch.cuh"
 
 namespace p3 {
@@ -402,51 +403,7 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
 // column kernel's ZYX-store form.  A wait that gives up sets bit 2 of
 // *a.err, waits (bounded) for the copies in flight and leaves the tile.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ bool mbar_try_wait(unsigned bar, unsigned parity)
-{
-    unsigned done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return done != 0;
-}
-
 constexpr int kTmaRows = 256;  // box height (elements of a line)
-
-// Copy barrier of a tile: arrival count 1, or 2 in the test mode of
-// StageArgs::wait_extra (one arrival never comes, so the wait runs out).
-__device__ __forceinline__ void copy_bar_init(unsigned bar, int extra)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(extra ? 2 : 1) : "memory");
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-}
-
-// Every thread waits (at most a.spin polls) for the tile's copies; true when
-// all threads saw them land.  Otherwise bit 2 of *a.err is set, the missing
-// test-mode arrival is supplied, and the CTA waits (again bounded) for the
-// copies still in flight into its shared memory before the caller leaves.
-__device__ __forceinline__ bool copy_bar_wait(const StageArgs& a, unsigned bar)
-{
-    int ok = 0;
-    for (unsigned it = 0; it < a.spin; ++it)
-        if (mbar_try_wait(bar, 0)) {
-            ok = 1;
-            break;
-        }
-    if (__syncthreads_and(ok)) return true;
-    if (threadIdx.x == 0) {
-        atomicOr(a.err, 2u);
-        if (a.wait_extra) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
-    }
-    __syncthreads();
-    for (unsigned it = 0; it < a.spin && !mbar_try_wait(bar, 0); ++it) {
-    }
-    return false;
-}
 
 template <int N, int SYM> __host__ __device__ constexpr int tma_rows()
 {

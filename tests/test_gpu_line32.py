@@ -62,3 +62,27 @@ def test_in_place_rows(shape):
     assert torch.equal(X, Xr)
     y = plan.backward(X, out=plan.real_view(X))[:, :, :nx]
     assert torch.equal(y, ref.backward(Xr))
+
+
+@pytest.mark.parametrize("shape", [(384, 60, 384), (190, 93, 486), (4094, 91, 24), (102, 41, 2000)])
+def test_bulk_copied_lines(shape):
+    """Inverse Z stage of the ZYX layout whose tile arrives line by line by bulk
+    copies: bit for bit the plan with P3_FLAG_NO_TMA; a wait that runs out is
+    reported."""
+    import torch
+    from paper_1905_02803_gb300 import p3dfft as P
+    pt = P.Plan(*shape, precision="f32")
+    pn = P.Plan(*shape, precision="f32", flags=P.P3_FLAG_NO_TMA)
+    assert "line32_bulk" in pt.describe() and "line32_bulk" not in pn.describe(), pt.describe()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(shape[0])
+    G = torch.view_as_complex(torch.randn(pt.complex_shape + (2,), generator=g, device="cuda"))
+    y = pt.backward(G)
+    assert torch.equal(y, pn.backward(G))
+    assert P.p3_plan_wait_status(pt.handle) == P.P3_OK
+    P.p3_plan_set_wait_limits(pt.handle, 2000, 1)
+    pt.backward(G)
+    assert P.p3_plan_wait_flags(pt.handle) == P.P3_WAIT_COPY
+    P.p3_plan_set_wait_limits(pt.handle, 1 << 23, 0)
+    assert torch.equal(y, pt.backward(G))
+    assert P.p3_plan_wait_status(pt.handle) == P.P3_OK
