@@ -326,6 +326,10 @@ class Plan:
         self._hook = None       # (python function, ctypes callback) while a Z hook is set
         self._bufs = {}         # device pointer -> tensor, for the current call
         self._hook_error = None
+        # looked up once: a call on a small grid takes longer to issue than to run
+        self._real_shape = (self.nz, self.ny, 2 * self.H if self.padded else self.nx)
+        self._complex_shape = (self.nz, self.ny, self.H) if layout == "xyz" else (self.H, self.ny, self.nz)
+        self._raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
     def __del__(self):
         h = getattr(self, "handle", None)
@@ -336,11 +340,11 @@ class Plan:
     @property
     def real_shape(self):
         """(nz, ny, nx), or (nz, ny, 2H) with padded real rows."""
-        return (self.nz, self.ny, 2 * self.H if self.padded else self.nx)
+        return self._real_shape
 
     @property
     def complex_shape(self):
-        return (self.nz, self.ny, self.H) if self.layout == "xyz" else (self.H, self.ny, self.nz)
+        return self._complex_shape
 
     def empty_real(self):
         return self.torch.empty(self.real_shape, dtype=self.real_dtype, device=self.device)
@@ -388,11 +392,23 @@ class Plan:
         self._hook = (fn, cb)
 
     def _call(self, c_fn, inp, out, ws, stream):
+        """Runs one transform (the library's p3_ftran_r2c or p3_btran_c2r)."""
+        if stream is not None:
+            s = stream.cuda_stream
+        elif self._raw_stream is not None:
+            s = self._raw_stream(self.device.index)
+        else:
+            s = self.torch.cuda.current_stream(self.device).cuda_stream
+        w = None if ws is None else ws.data_ptr()
+        if self._hook is None:
+            st = c_fn(self.handle, inp.data_ptr(), out.data_ptr(), w, s)
+            if st != P3_OK:
+                raise P3Error(st, c_fn.__name__)
+            return
         self._bufs = {t.data_ptr(): t for t in (ws, out) if t is not None}
         self._hook_error = None
         try:
-            st = c_fn(self.handle, inp.data_ptr(), out.data_ptr(), None if ws is None else ws.data_ptr(),
-                      self._stream(stream), check=False)
+            st = c_fn(self.handle, inp.data_ptr(), out.data_ptr(), w, s)
         finally:
             self._bufs = {}
         if st == P3_ERR_HOOK and self._hook_error is not None:
@@ -402,20 +418,19 @@ class Plan:
     def launches(self, direction: int) -> int:
         return p3_plan_launches(self.handle, direction)
 
-    def _stream(self, stream):
-        s = stream if stream is not None else self.torch.cuda.current_stream(self.device)
-        return ctypes.c_void_p(s.cuda_stream)
-
     def _check_tensor(self, t, shape, dtype, what):
-        if t.device != self.device or t.dtype != dtype or tuple(t.shape) != tuple(shape) or not t.is_contiguous():
+        if t.dtype != dtype or t.shape != shape or t.device != self.device or not t.is_contiguous():
             raise ValueError("%s must be a contiguous %s tensor of shape %s on %s" % (what, dtype, shape, self.device))
 
     def forward(self, x, out=None, ws=None, stream=None):
-        self._check_tensor(x, self.real_shape, self.real_dtype, "input")
-        out = self.empty_complex() if out is None else out
-        self._check_tensor(out, self.complex_shape, self.complex_dtype, "output")
-        ws = self.workspace() if ws is None else ws
-        self._call(p3_ftran_r2c, x, out, ws, stream)
+        self._check_tensor(x, self._real_shape, self.real_dtype, "input")
+        if out is None:
+            out = self.empty_complex()
+        else:
+            self._check_tensor(out, self._complex_shape, self.complex_dtype, "output")
+        if ws is None and self.ws_bytes:
+            ws = self.workspace()
+        self._call(_lib.p3_ftran_r2c, x, out, ws, stream)
         return out
 
     def complex_view(self, x):
@@ -427,11 +442,14 @@ class Plan:
         return self.torch.view_as_real(X).view(self.nz, self.ny, 2 * self.H)
 
     def backward(self, X, out=None, ws=None, stream=None):
-        self._check_tensor(X, self.complex_shape, self.complex_dtype, "input")
-        out = self.empty_real() if out is None else out
-        self._check_tensor(out, self.real_shape, self.real_dtype, "output")
-        ws = self.workspace() if ws is None else ws
-        self._call(p3_btran_c2r, X, out, ws, stream)
+        self._check_tensor(X, self._complex_shape, self.complex_dtype, "input")
+        if out is None:
+            out = self.empty_real()
+        else:
+            self._check_tensor(out, self._real_shape, self.real_dtype, "output")
+        if ws is None and self.ws_bytes:
+            ws = self.workspace()
+        self._call(_lib.p3_btran_c2r, X, out, ws, stream)
         return out
 
 
