@@ -99,6 +99,7 @@ struct PassConsts {
     int dq, dr;   // tpl / Ns, tpl mod Ns (a thread's step through the butterflies)
     unsigned pm;  // t / Ns = (t * pm) >> ps (see line_magic)
     int ps;
+    int toff;     // offset of the pass in a table of pass twiddles (pass_twiddles)
 };
 
 struct StageArgs {
@@ -126,7 +127,9 @@ struct StageArgs {
     const void* tw;    // tw[k] = exp(-2 pi i k / twn), complex of the stage type
     int twn;
     const void* tw2;   // real-split twiddles exp(-2 pi i k / Nx) (R2C/C2R_HALF), length Nx
-    const void* twr;   // power-of-two lines: per-pass twiddles laid out for row-style lanes
+    const void* twr;   // per-pass twiddles laid out for lanes with consecutive butterflies: power-of-two
+                       // lines for row-style lanes (p3_pow2.cuh); KIND_LINE32: pass p >= 1 holds at
+                       // pc[p].toff + (r - 1) Ns + q the entry q r tstep of tw
     // Bluestein (nfft not 7-smooth): DFT_nfft via padded length m
     int blue;
     int m;
@@ -160,8 +163,11 @@ struct StageArgs {
 inline void pass_consts(PassConsts* pc, int n, int npass, const int* rad, int tpl, int ts)
 {
     long long ns = 1;
+    int off = 0;
     for (int p = 0; p < npass && p < kMaxPasses; ++p) {
         const long long R = rad[p] > 0 ? rad[p] : 1;
+        pc[p].toff = off;
+        if (p > 0) off += (int)((R - 1) * ns);
         pc[p].tstep = (int)((n / (ns * R)) * ts);
         pc[p].dq = (int)(tpl / ns);
         pc[p].dr = (int)(tpl % ns);

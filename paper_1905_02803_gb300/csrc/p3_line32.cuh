@@ -12,13 +12,16 @@
 // and read HBM straight into the first pass.  The arithmetic is the same
 // operation for operation, so the results are too.
 //
-// Measured (forward + inverse): 384^3 907 -> 730 us, 375 x 360 x 343 885 ->
-// 690 us, 24 mixed grids 2.49 -> 2.08 ms, 48 x 40 x 36 39 -> 27 us (replayed
-// graph).  Per complex point a strided stage of 384 issues 79 instructions
-// (112 before), a row stage 71 - 73.  What bounds them now: the L1 data pipe
-// (65 - 83 % busy: exchanges, row loads, twiddles) and the latency of the
-// tile's loads; 85 registers (three CTAs) or 512-thread CTAs were 5 - 10 %
-// slower.
+// Pass twiddles come from tables in the order that consecutive butterflies read
+// them (one sector per warp and value instead of up to one per lane).
+//
+// Measured (forward + inverse): 384^3 907 -> 689 us, 375 x 360 x 343 885 ->
+// 651 us, 24 mixed grids 2.49 -> 1.94 ms, 48 x 40 x 36 39 -> 25 us (replayed
+// graph).  Per complex point a strided stage of 384 issues 80 instructions
+// (112 before), a row stage about 80 (125).  What bounds them now: no single
+// unit (L1 data pipe 41 - 64 % busy, issue about 50 %); the rest waits for the
+// tile's loads and the block barriers.  85 registers (three CTAs) were 5 - 10 %
+// slower, 512-thread CTAs throughout 7 %.
 #pragma once
 
 #include "p3_copy.cuh"
@@ -139,7 +142,7 @@ __device__ __forceinline__ void pass(const StageArgs& a, C* s, const Shared& sh,
             }
         }
     } else {
-        const C* tw = static_cast<const C*>(a.tw);
+        const C* tw = static_cast<const C*>(a.twr) + c.toff;
         int rr = r0;
 #pragma unroll
         for (int b = 0; b < BM; ++b) {
@@ -165,12 +168,11 @@ __device__ __forceinline__ void pass(const StageArgs& a, C* s, const Shared& sh,
             }
             if constexpr (!FIRST) {
                 if (rr) {
-                    const int k = rr * c.tstep;
-                    int idx = k;
+                    const C* tp = tw + rr;
 #pragma unroll
                     for (int r = 1; r < R; ++r) {
-                        v[b * R + r] = mul(v[b * R + r], ldg(tw + idx));
-                        idx += k;
+                        v[b * R + r] = mul(v[b * R + r], ldg(tp));
+                        tp += Ns;
                     }
                 }
                 if (b + 1 < BM) {
@@ -437,7 +439,7 @@ __device__ __forceinline__ void row_pass(const StageArgs& a, C* s, const Row& th
             }
         }
     } else {
-        const C* tw = static_cast<const C*>(a.tw);
+        const C* tw = static_cast<const C*>(a.twr) + c.toff;
         int rr = r0;
 #pragma unroll
         for (int b = 0; b < BM; ++b) {
@@ -445,12 +447,11 @@ __device__ __forceinline__ void row_pass(const StageArgs& a, C* s, const Row& th
 #pragma unroll
             for (int r = 0; r < R; ++r) v[b * R + r] = s[rslot(j + r * nb, ps)];
             if (rr) {
-                const int k = rr * c.tstep;
-                int idx = k;
+                const C* tp = tw + rr;
 #pragma unroll
                 for (int r = 1; r < R; ++r) {
-                    v[b * R + r] = mul(v[b * R + r], ldg(tw + idx));
-                    idx += k;
+                    v[b * R + r] = mul(v[b * R + r], ldg(tp));
+                    tp += Ns;
                 }
             }
             if (b + 1 < BM) {

@@ -46,7 +46,7 @@ struct Stage {
 };
 
 struct TableKey {
-    int kind;  // 0 roots, 1 chirp, 2 bhat, 3 row-style roots, 4 fixed-point roots
+    int kind;  // 0 roots, 1 chirp, 2 bhat, 3 row-style roots, 4 fixed-point roots, 5 pass twiddles
     long long n, m;
     bool operator<(const TableKey& o) const
     {
@@ -66,6 +66,7 @@ struct p3_plan_s {
     int device;
     size_t csize;  // bytes per complex element
     void* dtab;
+    std::vector<void*> tables;  // further device tables (tuned radix orders)
     // st[0] forward, st[1] inverse, st[2] the inverse used while a Z hook is
     // set (EMPTY third dimension: a Z copy into the work buffer comes first)
     std::vector<Stage> st[3];
@@ -288,6 +289,11 @@ long long pow2_ceil(long long v)
 struct TableSet {
     std::map<TableKey, size_t> offs;  // byte offsets into the device block
     std::vector<std::complex<double>> vals;
+    size_t find(const TableKey& k) const
+    {
+        auto it = offs.find(k);
+        return it == offs.end() ? (size_t)-1 : it->second;
+    }
     size_t add(const TableKey& k, std::vector<std::complex<double>>&& v)
     {
         auto it = offs.find(k);
@@ -301,6 +307,8 @@ struct TableSet {
 
 size_t roots_table(TableSet& T, long long n)
 {
+    const size_t have = T.find(TableKey{0, n, 0});
+    if (have != (size_t)-1) return have;
     std::vector<std::complex<double>> v((size_t)n);
     for (long long k = 0; k < n; ++k) v[(size_t)k] = unit_root(k, n);
     return T.add(TableKey{0, n, 0}, std::move(v));
@@ -309,6 +317,8 @@ size_t roots_table(TableSet& T, long long n)
 // the same for the FP64 fixed-point kernels
 size_t fixed_roots_table(TableSet& T, long long n)
 {
+    const size_t have = T.find(TableKey{4, n, 0});
+    if (have != (size_t)-1) return have;
     std::vector<std::complex<double>> v((size_t)n);
     for (long long k = 0; k < n; ++k) v[(size_t)k] = fixed_root(k, n);
     return T.add(TableKey{4, n, 0}, std::move(v));
@@ -339,6 +349,31 @@ size_t row_tw_table(TableSet& T, long long n, int E, long long tn)
         ns *= R;
     }
     return T.add(TableKey{3, n * 64 + E, tn}, std::move(v));
+}
+
+// Twiddles of the passes of a radix sequence over n points (StageArgs::twr of the
+// FP32 line kernels): pass p >= 1 stores, at (r - 1) Ns + q after the passes before
+// it, the entry q r tn / (Ns R) of the table of tn roots.
+std::vector<std::complex<double>> pass_twiddles(int npass, const int* rad, const std::complex<double>* roots, long long tn)
+{
+    std::vector<std::complex<double>> v;
+    long long ns = 1;
+    for (int p = 0; p < npass; ++p) {
+        const long long R = rad[p];
+        if (p >= 1) {
+            const long long step = tn / (ns * R);
+            for (long long r = 1; r < R; ++r)
+                for (long long q = 0; q < ns; ++q) v.push_back(roots[(q * r * step) % tn]);
+        }
+        ns *= R;
+    }
+    return v;
+}
+size_t pass_twiddle_table(TableSet& T, int npass, const int* rad, size_t roots, long long tn)
+{
+    long long code = 0;
+    for (int p = 0; p < npass; ++p) code = code * 17 + rad[p];
+    return T.add(TableKey{5, code, tn}, pass_twiddles(npass, rad, &T.vals[roots], tn));
 }
 
 size_t chirp_table(TableSet& T, long long n)
@@ -712,11 +747,31 @@ static p3_status tune_generic(p3_plan P, std::string& report)
             }
             float best = 1e30f;
             StageArgs pick = a0;
+            // a line kernel's pass twiddles follow the radix order: one table
+            // per candidate order, the picked one kept by the plan
+            const bool tabled = a0.kern == p3::KIND_LINE32;
+            std::vector<void*> tables;
             std::string line = std::string(d == 0 ? "fwd " : "bwd ") + st.name + " tuned:";
             for (const auto& o : orders) {
+                if (tabled && rc == P3_OK) {
+                    std::vector<std::complex<double>> roots((size_t)a0.twn);
+                    for (int k = 0; k < a0.twn; ++k) roots[(size_t)k] = unit_root(k, a0.twn);
+                    const std::vector<std::complex<double>> w = pass_twiddles((int)o.size(), o.data(), roots.data(), a0.twn);
+                    std::vector<float> host;
+                    for (const auto& z : w) {
+                        host.push_back((float)z.real());
+                        host.push_back((float)z.imag());
+                    }
+                    void* t = NULL;
+                    if (cudaMalloc(&t, host.size() * sizeof(float)) != cudaSuccess) rc = P3_ERR_NOMEM;
+                    else if (cudaMemcpy(t, host.data(), host.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)
+                        rc = P3_ERR_CUDA;
+                    tables.push_back(t);
+                }
                 for (int shrink = 0; shrink < 3 && rc == P3_OK; ++shrink) {
                     StageArgs a = a0;
                     for (size_t k = 0; k < o.size(); ++k) a.rad[k] = o[k];
+                    if (tabled) a.twr = tables.back();
                     if (a0.kern == p3::KIND_FIX64) {
                         if (!p3::fix64_configure(a, shrink)) break;
                     } else if (a0.kern == p3::KIND_LINE32) {
@@ -758,6 +813,10 @@ static p3_status tune_generic(p3_plan P, std::string& report)
                         pick = a;
                     }
                 }
+            }
+            for (void* t : tables) {
+                if (rc == P3_OK && t == pick.twr) P->tables.push_back(t);
+                else if (t) cudaFree(t);
             }
             if (rc != P3_OK) break;
             pick.src = NULL;
@@ -908,6 +967,7 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
             a.npass = 0;
         }
         tile_setup(a, P->csize, flags, !fx.empty());
+        if (a.kern == p3::KIND_LINE32) pd.twr = pass_twiddle_table(T, a.npass, a.rad, pd.tw - 1, a.twn) + 1;
         Stage s;
         s.a = a; s.src = src; s.dst = dst; s.name = name; s.bytes = bytes;
         s.fused = false;
@@ -1174,6 +1234,7 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
     if (flags & P3_FLAG_TUNE) {
         rc = tune_generic(P, tuned);
         if (rc != P3_OK) {
+            for (void* t : P->tables) cudaFree(t);
             if (P->dtab) cudaFree(P->dtab);
             if (P->derr) cudaFree(P->derr);
             cudaGetLastError();
@@ -1190,6 +1251,7 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
     if ((flags & P3_FLAG_TUNE) && any_fused) {
         rc = tune(P, unfused, tuned);
         if (rc != P3_OK) {
+            for (void* t : P->tables) cudaFree(t);
             if (P->dtab) cudaFree(P->dtab);
             if (P->derr) cudaFree(P->derr);
             cudaGetLastError();
@@ -1286,6 +1348,7 @@ p3_status p3_plan_destroy(p3_plan plan)
         cudaGetDevice(&cur);
         if (cur != plan->device) cudaSetDevice(plan->device);
         cudaFree(plan->derr);
+        for (void* t : plan->tables) cudaFree(t);
         if (cur >= 0 && cur != plan->device) cudaSetDevice(cur);
         cudaGetLastError();
     }
