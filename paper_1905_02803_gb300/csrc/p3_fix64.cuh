@@ -8,11 +8,12 @@
 // with one exponent per line (block floating point): a butterfly addition is
 // two 32-bit additions, a multiplication by a 64-bit twiddle part three
 // 32 x 32 -> 64 multiply-adds.  Doubles appear only in HBM.  Measured against
-// the double kernels (forward + inverse): 32^3 145 -> 45 us, 243 x 250 x 180
-// 2450 -> 803 us, 512^3 22.6 -> 7.0 ms in a first form.  What bounds them now
-// (256^3): issue slots 40-50 % busy, the rest waits for instruction fetch
-// (long unrolled passes), the double conversions and the dependent chains of
-// 16 to 32 warps per SM.
+// the double kernels: 32^3 forward + inverse 145 -> 31 us, 243 x 250 x 180 2450 ->
+// 764 us; inverse of 512^3 11.2 -> 3.1 ms (stages 3.45 / 3.45 / 4.27 -> 0.89 /
+// 0.87 / 1.33 ms), of the 480 x 360 x 257 channel grid 5.3 -> 1.4 ms.  What bounds
+// them now: issue slots 40-50 % busy, the rest waits for instruction fetch (long
+// unrolled passes), the double conversions and the dependent chains of 16 to 32
+// warps per SM.
 //
 // Precision.  A line is aligned to its largest component: |v| < 2^58, so the
 // quantum is at least 2^-58 of that component, 2^5 finer than the last bit of
@@ -628,8 +629,28 @@ __device__ __forceinline__ void pass(const StageArgs& a, Q* s, Shared& sh, Threa
             }
         } else {
             // Z[k] = X1[k] + i X2[k], Z[n-k] = conj X1[k] + i conj X2[k]
-            // (k >= 1); imaginary parts of X1[0], X2[0] dropped; swapped
+            // (k >= 1); imaginary parts of X1[0], X2[0] dropped; swapped.  One
+            // thread per pair of bins, in place: X1[k] sits at slot k and X2[k] at
+            // H + k, where Z[k] and Z[n-k] take their places.
             const int H = a.n_in;
+            if (th.valid) {
+                for (int k = t; k < H; k += tpl) {
+                    Q f = s[k * LDB + l], h = s[(H + k) * LDB + l];
+                    if (tiny && mw) {
+                        f = Q{scaled(f.x), scaled(f.y)};
+                        h = Q{scaled(h.x), scaled(h.y)};
+                    }
+                    Q A = Q{to_fix<AL>(f.x, emax), to_fix<AL>(f.y, emax)};
+                    Q C = Q{to_fix<AL>(h.x, emax), to_fix<AL>(h.y, emax)};
+                    if (k == 0) {
+                        A.y = 0;
+                        C.y = 0;
+                    }
+                    s[k * LDB + l] = Q{A.y + C.x, A.x - C.y};
+                    s[(H + k) * LDB + l] = Q{C.x - A.y, A.x + C.y};
+                }
+            }
+            __syncthreads();
 #pragma unroll
             for (int b = 0; b < BM; ++b) {
                 const int j = t + b * tpl;
@@ -637,29 +658,11 @@ __device__ __forceinline__ void pass(const StageArgs& a, Q* s, Shared& sh, Threa
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     const int e = j + r * nb;
-                    Q z = Q{0, 0};
-                    if (ok) {
-                        const bool up_half = e < H;
-                        const int k = up_half ? e : n - e;
-                        Q f = s[k * LDB + l], h = s[(H + k) * LDB + l];
-                        if (tiny && mw) {
-                            f = Q{scaled(f.x), scaled(f.y)};
-                            h = Q{scaled(h.x), scaled(h.y)};
-                        }
-                        Q A = Q{to_fix<AL>(f.x, emax), to_fix<AL>(f.y, emax)};
-                        Q C = Q{to_fix<AL>(h.x, emax), to_fix<AL>(h.y, emax)};
-                        if (k == 0) {
-                            A.y = 0;
-                            C.y = 0;
-                        }
-                        z = up_half ? Q{A.y + C.x, A.x - C.y} : Q{C.x - A.y, A.x + C.y};
-                    }
-                    v[b * R + r] = z;
+                    v[b * R + r] = ok ? s[(e < H ? e : H + n - e) * LDB + l] : Q{0, 0};
                 }
             }
-            __syncthreads();  // every thread has read the staged slots
         }
-        if constexpr (K == K_C2R) __syncthreads();
+        if constexpr (K == K_C2R || K == K_CP) __syncthreads();  // every thread has read its values
         th.sexp = sexp;
         th.bad = bad;
     } else {
