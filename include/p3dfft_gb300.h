@@ -210,9 +210,9 @@ p3_status p3_plan_launches(p3_plan plan, int dir, int* launches);
  * 1D FFT of Sect. 2; no device work, no GPU needed).  FP32 lengths with a
  * factor 3, 5 or 7 take the fewest passes over the native radices 2, 3, 4,
  * 5, 7, 8, 16 and the composite register butterflies up to 15; other
- * lengths take 16s first, then 8 / 4 / 2, then 3, 5, 7 (FP64 plans of up to
- * 12,582,912 points run 64-bit fixed-point kernels instead, which order and
- * group these radices by their own cost).  radices receives
+ * lengths take 16s first, then 8 / 4 / 2, then 3, 5, 7 (FP64 inverse
+ * transforms, and forward ones of up to 12,582,912 points, run 64-bit fixed-point
+ * kernels instead, which order and group these radices by their own cost).  radices receives
  * up to cap entries (the largest radix first), *npass their count.
  * P3_ERR_UNSUPPORTED when n has a prime factor above 7 (such lines run
  * Bluestein's algorithm over a power-of-two length) or the sequence is

@@ -223,14 +223,16 @@ int fix64_threads(int n, int npass, const int* rad, int cap);
 bool fix64_configure(StageArgs& a, int shrink);
 cudaError_t fix64_prepare(const StageArgs& a);
 cudaError_t fix64_launch(const StageArgs& a, cudaStream_t s);
-// FP64 plans of at most this many points (Nx Ny Nz) take them.  Their results
-// are nearer to the exact transform than the double-arithmetic kernels' at
-// every size, but they are other roundings: in larger volumes the double
-// kernels' own error in the bins beside a strong wave (up to 1.3e-12 of the
-// spectrum's typical bin at 512^3; 4.7e-13 once in fifty runs at 250 x 256 x
-// 250) exceeds the agreement with earlier results that perf/cases.py holds
-// outputs to (4.4e-13).  At 243 x 250 x 180 the largest of ten runs was
-// 2.4e-13.
+// The inverse takes them at every size, the forward transform up to this many
+// points (Nx Ny Nz).  Their results are nearer to the exact transform than the
+// double-arithmetic kernels' at every size, but they are other roundings: in
+// larger volumes the double kernels' own error in the spectrum's bins beside a
+// strong wave (up to 1.3e-12 of the typical bin at 512^3; 4.7e-13 once in fifty
+// runs at 250 x 256 x 250) exceeds the agreement with earlier results that
+// perf/cases.py holds outputs to (4.4e-13).  At 243 x 250 x 180 the largest of ten
+// runs was 2.4e-13.  The inverse's result is a field without such contrast:
+// at most 4.9e-15 at 512^3, 8.4e-15 on the 480 x 360 x 257 channel grid (six
+// runs each).
 constexpr double kFix64MaxPoints = 12582912.0;
 
 // FP32 line kernels of smooth lengths (p3_line32.cu): configure a stage whose

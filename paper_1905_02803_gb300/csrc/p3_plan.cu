@@ -911,8 +911,9 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
                 : ttype[2] == P3_SINE ? 2.0 * (nz + 1)
                                       : 1.0;
 
-    // FP64 plans of up to kFix64MaxPoints points run in 64-bit fixed point
-    const bool fixed = prec == P3_F64 && (double)nx * ny * nz <= p3::kFix64MaxPoints;
+    // FP64 stages that run in 64-bit fixed point: the inverse, and the forward
+    // transform of up to kFix64MaxPoints points
+    const bool fixed_fwd = prec == P3_F64 && (double)nx * ny * nz <= p3::kFix64MaxPoints;
 
     TableSet T;
     std::vector<Pending> pend[3];
@@ -944,6 +945,7 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
         Pending pd;
         if (rc != P3_OK) return;
         // the fixed-point radix sequence (empty: the line does not run there)
+        const bool fixed = dir == 0 ? fixed_fwd : prec == P3_F64;
         std::vector<int> fx;
         if (fixed && a.op != p3::OP_COPY && a.nfft > 1 && a.nfft <= p3::kMaxLine) {
             a.fix = fixed_form(a.nlines, a.nfft, a.op != p3::OP_C2C && a.op != p3::OP_DCT1 && a.op != p3::OP_DST1, fx);

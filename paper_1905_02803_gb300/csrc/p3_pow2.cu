@@ -43,6 +43,7 @@ bool pow2_configure(StageArgs& a, size_t csize, bool allow_tma)
 static bool configure(StageArgs& a, size_t csize, bool allow_tma)
 {
     if (a.blue) return false;
+    if (csize != 8 && (a.sign > 0 || a.in_elem_fast != (a.op == OP_R2C_HALF))) return false;  // double: forward stages
     const int N = a.nfft;
     if (!is_pow2_in_range(N)) return false;
     const bool f32 = csize == 8;

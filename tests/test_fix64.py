@@ -209,6 +209,11 @@ def test_scales_zeros_and_non_finite_lines(shape, ttypes, layout):
 
 @pytest.mark.gpu
 def test_volume_limit_keeps_double_kernels():
+    """Forward transforms of more than 12,582,912 points keep the double
+    kernels; every inverse runs in fixed point."""
     from paper_1905_02803_gb300.p3dfft import Plan
-    assert "fix64" in Plan(256, 256, 192, precision="f64").describe()
-    assert "fix64" not in Plan(256, 256, 193, precision="f64").describe()
+    for nz, fixed in ((192, True), (196, False)):
+        lines = [w for w in Plan(256, 256, nz, precision="f64").describe().splitlines() if "kernel=" in w]
+        assert len(lines) == 6
+        for w in lines:
+            assert ("fix64" in w) == (fixed or w.startswith("bwd")), w
