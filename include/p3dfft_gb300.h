@@ -319,7 +319,8 @@ p3_status p3_plan_set_z_hook(p3_plan plan, p3_z_hook fn, void* user);
  *     graph.  Results equal each plan's own within rounding (the power-of-two
  *     and plane-fused kernels a plan may use alone are not used here).
  *   Streams (nstreams >= 1): the plans' own launches spread over nstreams
- *     internal streams (largest plans first, each to the least loaded
+ *     internal streams, or four if that is less and the grids average 3 M
+ *     points or more (largest plans first, each to the least loaded
  *     stream), so the launches of different plans overlap on the GPU;
  *     results equal each plan's own bit for bit.
  *
