@@ -99,7 +99,6 @@ struct PassConsts {
     int dq, dr;   // tpl / Ns, tpl mod Ns (a thread's step through the butterflies)
     unsigned pm;  // t / Ns = (t * pm) >> ps (see line_magic)
     int ps;
-    int toff;     // offset of the pass in a table of pass twiddles (pass_twiddles)
 };
 
 struct StageArgs {
@@ -108,6 +107,10 @@ struct StageArgs {
     // call's source pointer
     CUtensorMap tmap;
     const void* src;
+    // (the persistent batch copies what follows dst for every task)
+    int fix;           // KIND_FIX64: which of its kernels (32 fx::Kind + largest radix); KIND_LINE32: l32::Kind
+    // KIND_LINE32 with bulk copies: slots between the input lines
+    int box;
     void* dst;
     LineMap in, out;
     long long nlines;
@@ -129,7 +132,7 @@ struct StageArgs {
     const void* tw2;   // real-split twiddles exp(-2 pi i k / Nx) (R2C/C2R_HALF), length Nx
     const void* twr;   // per-pass twiddles laid out for lanes with consecutive butterflies: power-of-two
                        // lines for row-style lanes (p3_pow2.cuh); KIND_LINE32: pass p >= 1 holds at
-                       // pc[p].toff + (r - 1) Ns + q the entry q r tstep of tw
+                       // (r - 1) Ns + q, after the passes before it, the entry q r tstep of tw
     // Bluestein (nfft not 7-smooth): DFT_nfft via padded length m
     int blue;
     int m;
@@ -143,13 +146,10 @@ struct StageArgs {
     size_t smem;       // dynamic shared memory bytes
     int threads;       // B * tpl
     int kern;          // KernelKind
-    int fix;           // KIND_FIX64: which of its kernels (32 fx::Kind + largest radix); KIND_LINE32: l32::Kind
     // 1: tensor-core split-precision kernel (p3_tc.cu)
     int tc;
     // 1: input tile by tensor copies (tmap); 2: by bulk copies
     int tma;
-    // KIND_LINE32 with bulk copies: slots between the input lines
-    int box;
     // status word of the plan: a bounded device wait that gave up ORs a bit in
     unsigned* err;
     // polls before a wait for a tensor / bulk copy gives up
@@ -163,11 +163,8 @@ struct StageArgs {
 inline void pass_consts(PassConsts* pc, int n, int npass, const int* rad, int tpl, int ts)
 {
     long long ns = 1;
-    int off = 0;
     for (int p = 0; p < npass && p < kMaxPasses; ++p) {
         const long long R = rad[p] > 0 ? rad[p] : 1;
-        pc[p].toff = off;
-        if (p > 0) off += (int)((R - 1) * ns);
         pc[p].tstep = (int)((n / (ns * R)) * ts);
         pc[p].dq = (int)(tpl / ns);
         pc[p].dr = (int)(tpl % ns);

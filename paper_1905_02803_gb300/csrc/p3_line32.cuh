@@ -103,7 +103,7 @@ struct Thread {
 // BULK: the input tile came line by line by bulk copies, element e of line l at
 // l * a.box + e.
 template <int K, bool BULK, int R, bool FIRST>
-__device__ __forceinline__ void pass(const StageArgs& a, C* s, const Shared& sh, const Thread& th, int p, int Ns)
+__device__ __forceinline__ void pass(const StageArgs& a, C* s, const Shared& sh, const Thread& th, int p, int Ns, int toff)
 {
     constexpr int BM = bfly<R>();
     const int n = a.nfft, nb = n / R, tpl = a.tpl, LDB = a.LDB;
@@ -142,7 +142,7 @@ __device__ __forceinline__ void pass(const StageArgs& a, C* s, const Shared& sh,
             }
         }
     } else {
-        const C* tw = static_cast<const C*>(a.twr) + c.toff;
+        const C* tw = static_cast<const C*>(a.twr) + toff;
         int rr = r0;
 #pragma unroll
         for (int b = 0; b < BM; ++b) {
@@ -254,11 +254,12 @@ __device__ __forceinline__ void pass(const StageArgs& a, C* s, const Shared& sh,
 }
 
 template <int K, bool BULK, bool FIRST>
-__device__ __forceinline__ void pass_any(const StageArgs& a, C* s, const Shared& sh, const Thread& th, int p, int Ns)
+__device__ __forceinline__ void pass_any(const StageArgs& a, C* s, const Shared& sh, const Thread& th, int p, int Ns,
+                                         int toff)
 {
     switch (a.rad[p]) {
 #define P3_L32_PASS(R) \
-    case R: pass<K, BULK, R, FIRST>(a, s, sh, th, p, Ns); break;
+    case R: pass<K, BULK, R, FIRST>(a, s, sh, th, p, Ns, toff); break;
         P3_L32_PASS(2) P3_L32_PASS(3) P3_L32_PASS(4) P3_L32_PASS(5) P3_L32_PASS(6) P3_L32_PASS(7) P3_L32_PASS(8)
         P3_L32_PASS(9) P3_L32_PASS(10) P3_L32_PASS(12) P3_L32_PASS(14) P3_L32_PASS(15) P3_L32_PASS(16)
 #undef P3_L32_PASS
@@ -327,10 +328,11 @@ __global__ void __launch_bounds__(kThreadsMost, 2) kernel(const __grid_constant_
     th.t = tid >> lb;
     th.act = th.t < a.tpl;
     th.valid = th.act && th.l < rows;
-    pass_any<K, BULK, true>(a, s, sh, th, 0, 1);
-    int Ns = a.rad[0];
+    pass_any<K, BULK, true>(a, s, sh, th, 0, 1, 0);
+    int Ns = a.rad[0], toff = 0;  // toff: the pass's place in the table of pass twiddles
     for (int p = 1; p < a.npass; ++p) {
-        pass_any<K, BULK, false>(a, s, sh, th, p, Ns);
+        pass_any<K, BULK, false>(a, s, sh, th, p, Ns, toff);
+        toff += (a.rad[p] - 1) * Ns;
         Ns *= a.rad[p];
     }
 
@@ -376,7 +378,7 @@ struct Row {
 };
 
 template <int K, int R, bool FIRST>
-__device__ __forceinline__ void row_pass(const StageArgs& a, C* s, const Row& th, int p, int Ns)
+__device__ __forceinline__ void row_pass(const StageArgs& a, C* s, const Row& th, int p, int Ns, int toff)
 {
     constexpr int BM = bfly<R>();
     const int n = a.nfft, nb = n / R, tpl = a.tpl, t = th.t, ps = a.LDB;
@@ -439,7 +441,7 @@ __device__ __forceinline__ void row_pass(const StageArgs& a, C* s, const Row& th
             }
         }
     } else {
-        const C* tw = static_cast<const C*>(a.twr) + c.toff;
+        const C* tw = static_cast<const C*>(a.twr) + toff;
         int rr = r0;
 #pragma unroll
         for (int b = 0; b < BM; ++b) {
@@ -502,11 +504,11 @@ __device__ __forceinline__ void row_pass(const StageArgs& a, C* s, const Row& th
     if (!direct) __syncthreads();
 }
 
-template <int K, bool FIRST> __device__ __forceinline__ void row_any(const StageArgs& a, C* s, const Row& th, int p, int Ns)
+template <int K, bool FIRST> __device__ __forceinline__ void row_any(const StageArgs& a, C* s, const Row& th, int p, int Ns, int toff)
 {
     switch (a.rad[p]) {
 #define P3_L32_PASS(R) \
-    case R: row_pass<K, R, FIRST>(a, s, th, p, Ns); break;
+    case R: row_pass<K, R, FIRST>(a, s, th, p, Ns, toff); break;
         P3_L32_PASS(2) P3_L32_PASS(3) P3_L32_PASS(4) P3_L32_PASS(5) P3_L32_PASS(6) P3_L32_PASS(7) P3_L32_PASS(8)
         P3_L32_PASS(9) P3_L32_PASS(10) P3_L32_PASS(12) P3_L32_PASS(14) P3_L32_PASS(15) P3_L32_PASS(16)
 #undef P3_L32_PASS
@@ -540,10 +542,11 @@ template <int K> __global__ void __launch_bounds__(kThreadsMost, 2) row_kernel(c
     const int ps = a.LDB;
     C* sl = s + l * rpitch(n, ps);
     stage_begin();
-    row_any<K, true>(a, sl, th, 0, 1);
-    int Ns = a.rad[0];
+    row_any<K, true>(a, sl, th, 0, 1, 0);
+    int Ns = a.rad[0], toff = 0;
     for (int p = 1; p < a.npass; ++p) {
-        row_any<K, false>(a, sl, th, p, Ns);
+        row_any<K, false>(a, sl, th, p, Ns, toff);
+        toff += (a.rad[p] - 1) * Ns;
         Ns *= a.rad[p];
     }
     if constexpr (K == K_R2C) {
