@@ -855,7 +855,6 @@ template <typename T> __host__ __device__ constexpr int col_B(int N)
 // us) and keep 8.  The line lies at 64 KB between elements (Y: at most 32 KB
 // for rows of up to 4096 bins; Z of a 512-point plane 1 MB).
 constexpr int kWideB = 16;
-constexpr long long kWideStride = 65536 / 8;  // complex elements
 __host__ __device__ constexpr bool has_wide(int N) { return N == 512; }
 
 // Row-style ZYX-load kernel for FP32 lines of 256 .. 2048 points (a line's
