@@ -133,9 +133,11 @@ typedef enum { P3_LAYOUT_ZYX = 0, P3_LAYOUT_XYZ = 1 } p3_layout;
  *                second.
  *              P3_FLAG_NO_TMA: load the Z stages' input tiles with ordinary
  *                loads instead of tensor-memory-access (TMA) copies: the
- *                forward ZYX-store stage (FP32 lines of 256 .. 2048 points)
- *                and the inverse ZYX-load stage when its lines lie one after
- *                another in memory (FP32 FFT lines of 256 .. 1024 points).
+ *                forward ZYX-store stage and the XYZ Z stages (FP32 lines of
+ *                256 .. 2048 points), the inverse ZYX-load stage when its
+ *                lines lie one after another in memory (FP32 FFT lines of
+ *                256 .. 2048 points), and the inverse ZYX-load stage of large
+ *                FP32 volumes with even lines of other smooth lengths.
  * Any line length is accepted: lengths whose prime factors are 2, 3, 5, 7 run
  * natively; other lengths use Bluestein's chirp-z algorithm.  Lines longer
  * than 4096 points (2048 when Bluestein is needed) return P3_ERR_UNSUPPORTED.
@@ -154,7 +156,9 @@ p3_status p3_plan_destroy(p3_plan plan);
  * p3_ftran_r2c -- forward transform (R2C: X-pencil input, Z-pencil output,
  * Sect. 3.2).  in_real: Nx*Ny*Nz reals; out_cplx: H*Ny*Nz complex in the
  * plan's layout; workspace: p3_plan_workspace_bytes() bytes (may be NULL
- * when that is 0).  Errors: P3_ERR_INVALID (NULL plan/in/out, misaligned or
+ * when that is 0).  An infinity or a NaN in a line makes that line's transform
+ * non-finite (FP64 fixed-point stages: NaN throughout).
+ * Errors: P3_ERR_INVALID (NULL plan/in/out, misaligned or
  * partly overlapping buffers), P3_ERR_UNSUPPORTED (in == out without
  * P3_FLAG_PADDED_REAL), P3_ERR_WORKSPACE,
  * P3_ERR_CUDA (launch failure; the stream state is then undefined).

@@ -21,8 +21,9 @@
 // headroom (an OR over all magnitudes), so a pass loses only the bits that
 // the data really grew; twiddles carry 60 fractional bits and the butterfly
 // constants 64 (a double: 53).  The result is rounded once, to nearest, when
-// it becomes a double again.  Errors against a 113-bit reference are 2 - 4
-// times smaller than the double-arithmetic kernels' (see the tests).
+// it becomes a double again.  Relative errors of a forward + inverse pair
+// against a 64-bit reference: 3.5e-16 -> 2.7e-16 (32^3) and 6.0e-16 -> 3.7e-16
+// (243 x 250 x 180) from the double kernels to these.
 //
 // Bounds.  Components of |v| < 2^58 make complex moduli below 2^58.5; a
 // radix-R butterfly (R <= 16) and all its partial sums stay below
