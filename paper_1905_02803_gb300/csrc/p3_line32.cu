@@ -99,6 +99,12 @@ bool line32_configure(StageArgs& a, int shrink, bool allow_tma)
     if (tpl > l32::kThreadsMost) return false;
     if (k >= l32::K_R2C) {
         // rows: any number of lines per CTA
+        // Short even rows stay with the generic kernel, whose threads walk a tile's
+        // rows as one run: a row's one to three threads here read its values
+        // apart.  32 x 256 x 512: 58 us against 76; 60-point rows 53 against 57;
+        // 48 the same; 80-point rows 64 against 62.  Volumes below 2^20 values are
+        // bound by latency and run faster here (48 x 40 x 36: 25 us against 31).
+        if ((k == l32::K_R2C || k == l32::K_C2R) && n < 32 && a.nlines * n >= (1LL << 20)) return false;
         int B = tpl < l32::kThreads ? l32::kThreads / tpl : 1;
         const int ps = row_pad(n, a.npass, a.rad, tpl, B);
         const size_t row = (size_t)l32::rpitch(n, ps) * 8;
