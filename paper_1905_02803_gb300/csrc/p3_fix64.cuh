@@ -505,7 +505,10 @@ __device__ __forceinline__ void pass(const StageArgs& a, Q* s, Shared& sh, Threa
     Q v[BM * R];
 
     if constexpr (FIRST) {
-        unsigned m = 0;
+        // largest high word of the line's magnitudes; the low words only count as
+        // zero or not, so that a line of denormals below 2^-1042, whose high
+        // words are all 0, is told from a line of zeros
+        unsigned m = 0, low = 0;
         if constexpr (K != K_C2R && K != K_CP) {
             const ll es = a.in.es;
             const int M = n >> 1;
@@ -546,6 +549,7 @@ __device__ __forceinline__ void pass(const StageArgs& a, Q* s, Shared& sh, Threa
                 for (int i = b * R; i < b * R + R; ++i) {
                     m = max(m, hi_abs(v[i].x));
                     m = max(m, hi_abs(v[i].y));
+                    low |= (unsigned)v[i].x | (unsigned)v[i].y;
                 }
             }
         } else {
@@ -555,9 +559,14 @@ __device__ __forceinline__ void pass(const StageArgs& a, Q* s, Shared& sh, Threa
             for (int e = t; e <= n && th.valid; e += tpl) {
                 const Q x = s[e * LDB + l];
                 m = max(m, hi_abs(x.x));
-                if (e != 0 && e != d1) m = max(m, hi_abs(x.y));
+                low |= (unsigned)x.x;
+                if (e != 0 && e != d1) {
+                    m = max(m, hi_abs(x.y));
+                    low |= (unsigned)x.y;
+                }
             }
         }
+        if (low) m |= 1u;
         post<true>(m, sh.word, B, l);
         __syncthreads();
         const unsigned mw = sh.word[l];

@@ -208,6 +208,36 @@ def test_scales_zeros_and_non_finite_lines(shape, ttypes, layout):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("shape,z", [((24, 20, 18), "fft"), ((15, 12, 9), "fft"), ((15, 9, 17), "cheb"), ((32, 10, 15), "sine")])
+@pytest.mark.parametrize("layout", ["zyx", "xyz"])
+def test_lines_of_the_smallest_denormals(shape, z, layout):
+    """Values of a few units of 2^-1074: every stage's lines, sums included, lie
+    below 2^-1042, where a double's high word is zero.  Forward and inverse
+    equal the transform of the same whole numbers, times 2^-1074, but for the
+    rounding of each stage's results to whole units."""
+    import torch
+    from paper_1905_02803_gb300.p3dfft import Plan
+    nx, ny, nz = shape
+    plan = Plan(nx, ny, nz, precision="f64", ttypes=("fft", "fft", z), layout=layout)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(nx)
+    unit = 2.0 ** -537  # 2^-1074 in two steps, each exact
+    n = torch.randint(0, 16, plan.real_shape, generator=g, device="cuda").double()
+    m = torch.randint(0, 16, plan.complex_shape + (2,), generator=g, device="cuda").double()
+    got = torch.view_as_real(plan.forward(n * unit * unit)) / unit / unit
+    back = plan.backward(torch.view_as_complex(m * unit * unit)) / unit / unit
+    # a unit per stage (half by rounding to whole units, less by the rounding to
+    # 53 bits before it), in each part of a value; the transforms after it add up
+    # as many of them as their lines have points
+    zl = {"fft": nz, "cheb": 2 * (nz - 1), "sine": 2 * (nz + 1)}[z]
+    bound = 1.5 * (1 + zl + ny * zl)
+    boundb = 1.5 * (1 + nx + nx * ny)
+    want, wantb = torch.view_as_real(plan.forward(n)), plan.backward(torch.view_as_complex(m))
+    assert (got - want).abs().max().item() <= bound < 0.2 * want.abs().max().item()
+    assert (back - wantb).abs().max().item() <= boundb < 0.2 * wantb.abs().max().item()
+
+
+@pytest.mark.gpu
 def test_volume_limit_keeps_double_kernels():
     """Forward transforms of more than 12,582,912 points keep the double
     kernels; every inverse runs in fixed point."""
