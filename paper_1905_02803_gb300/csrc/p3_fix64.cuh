@@ -718,7 +718,6 @@ __device__ __forceinline__ void pass(const StageArgs& a, Q* s, Shared& sh, Threa
     }
 
     // positions (j / Ns) Ns R + j mod Ns + r Ns
-    if (last) stage_ending();
     if constexpr (!out_staged<K>()) {
         if (last) {
             const LineExp le = line_exp(th.sexp, th.bad);

@@ -184,8 +184,8 @@ inline void generic_consts(StageArgs& a)
 }
 
 // Launches a stage kernel that starts with stage_begin() (p3_launch.cuh): its
-// blocks may be resident, up to that point, while the stage before it in the
-// stream finishes.
+// blocks may be resident, up to that point, from when the last blocks of the
+// stage before it in the stream leave.
 inline cudaError_t launch_overlapped(void* fn, unsigned grid, unsigned block, void** args, size_t smem, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};

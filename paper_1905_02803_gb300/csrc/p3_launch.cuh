@@ -1,11 +1,18 @@
 // Overlap of a stage's launch with the end of the stage before it
 // (programmatic dependent launch): the next stage's launch latency, prologue
-// and first instruction fetches run while the last blocks of this one store
-// their results.  Measured, forward + inverse: 64^3 FP32 34.8 -> 26.6 us, 32^3
-// FP64 45.2 -> 30.8 us, 256^3 FP32 171 -> 156 us, 24 mixed grids over 16 streams
-// 2.08 -> 1.91 ms, 384^3 731 -> 720 us.  Letting the next blocks in from the
-// start of a stage instead parks them on SMs that other streams' stages, or the
-// stage's own last blocks, could use (128^3: 44 us against 38).
+// and first instruction fetches run while the last blocks of this one leave
+// and their writes become visible.  Forward + inverse without and with it, on
+// a stream: 64^3 FP32 37.0 -> 22.1 us, 32^3 FP64 48.2 -> 30.3, 256^3 FP32 169.2
+// -> 152.5, 384^3 701 -> 680; in a replayed graph, whose launches are cheaper,
+// 24.5 -> 21.8, 31.8 -> 30.5, 155.5 -> 151.8, 685 -> 679 us.
+//
+// No stage lets the next one in before its blocks leave
+// (griddepcontrol.launch_dependents): the blocks let in early go to the SMs
+// with room, not evenly, and then run there one after another, while other
+// SMs idle.  Measured with that call before each stage's stores: 64 x 64 x 256
+// FP32 24.5 -> 38.1 us, 64 x 64 x 512 34.2 -> 48.7, 112^3 FP64 XYZ 89 -> 102,
+// 1024 x 1024 x 3 XYZ 78 -> 95; it gained 1 to 3 us on cubes of 40, 80 and 135
+// points (41.4 -> 39.1 us), and over 444 calls it lost 5 % in FP32, 3 % in FP64.
 #pragma once
 
 namespace p3 {
@@ -17,14 +24,6 @@ __device__ __forceinline__ void stage_begin()
 {
 #if P3_PDL
     asm volatile("griddepcontrol.wait;" ::: "memory");
-#endif
-}
-// From here on (each block's outputs are computed) the next stage's blocks may
-// take free slots of the SMs, where they wait in stage_begin().
-__device__ __forceinline__ void stage_ending()
-{
-#if P3_PDL
-    asm volatile("griddepcontrol.launch_dependents;");
 #endif
 }
 

@@ -186,7 +186,6 @@ __device__ __forceinline__ void pass(const StageArgs& a, C* s, const Shared& sh,
 #pragma unroll
     for (int b = 0; b < BM; ++b) Dft<C, float, R>::run(v + b * R);
 
-    if (last) stage_ending();
     if constexpr (!out_staged<K>()) {
         if (last) {
             const ll es = a.out.es;
@@ -466,7 +465,6 @@ __device__ __forceinline__ void row_pass(const StageArgs& a, C* s, const Row& th
 #pragma unroll
     for (int b = 0; b < BM; ++b) Dft<C, float, R>::run(v + b * R);
 
-    if (last) stage_ending();
     const bool direct = last && (K == K_C2R || K == K_CP);
     if (!direct) __syncthreads();  // every thread has read its inputs
     int qq = q0, rr = r0;

@@ -241,9 +241,7 @@ template <> struct Vec4<float> { typedef float4 t; };
 // x[e - 1] below M and -x[N - 1 - e] above; output k is i times bin k + 1).
 // One tile of B lines (tile index `tile`, lines offset by `off` elements in
 // both arrays); s: the tile's shared memory.
-// STAGE: the tile is all that its block does of a stage (stage_ending).
-template <typename T, int N, int E, int B, int MODE, bool INV, int SYM, int LP = LD_DEF, int SP = ST_DEF,
-          bool STAGE = false>
+template <typename T, int N, int E, int B, int MODE, bool INV, int SYM, int LP = LD_DEF, int SP = ST_DEF>
 __device__ __forceinline__ void col_tile(const StageArgs& a, long long tile, long long off,
                                          typename CxT<T>::t* s)
 {
@@ -319,9 +317,6 @@ __device__ __forceinline__ void col_tile(const StageArgs& a, long long tile, lon
     }
     pass_compute<C, T, N, E, 0>(v, t, tw, 1);
     ColRest<C, T, N, E, B, SWZ, 1, NP>::run(v, s, l, t, tw);
-    // (in the 8-line strided kernels of 512 points and more the early call costs
-    // more than it hides: Y of 512^3 220 us with it, 214 without)
-    if constexpr (STAGE && (MODE != 0 || N < 512 || B >= 16)) stage_ending();
 
     typedef PassIdx<N, E, NP - 1> PLast;
     if constexpr (MODE != 1) {
@@ -389,7 +384,7 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     stage_begin();
-    col_tile<T, N, E, B, MODE, INV, SYM, LD_DEF, ST_DEF, true>(a, blockIdx.x, 0, reinterpret_cast<typename CxT<T>::t*>(smem_raw));
+    col_tile<T, N, E, B, MODE, INV, SYM>(a, blockIdx.x, 0, reinterpret_cast<typename CxT<T>::t*>(smem_raw));
 }
 
 // ---------------------------------------------------------------------------
@@ -472,7 +467,6 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
         }
     pass_compute<C, T, N, E, 0>(v, t, tw, 1);
     ColRest<C, T, N, E, B, ZYX, 1, NP>::run(v, s, l, t, tw);  // starts with a block barrier
-    if constexpr (N < 1024) stage_ending();  // longer tiles: costs more than it hides (1024^3: 4 us a stage)
 
     typedef PassIdx<N, E, NP - 1> PLast;
     if constexpr (!ZYX) {
@@ -589,7 +583,7 @@ template <class C, class T, int N, int E, int NP, int TS> struct RowRest<C, T, N
 };
 
 // Rows L0 .. L0 + B - 1 (those below Lend) of a row stage; s: the tile's
-// shared memory.
+// shared memory.  STAGE: all threads of the block work on this one tile.
 template <typename T, int N, int E, int B, int OPR, int LP = LD_DEF, int SP = ST_DEF, bool STAGE = false>
 __device__ __forceinline__ void row_tile(const StageArgs& a, long long L0, long long Lend, typename CxT<T>::t* s)
 {
@@ -636,7 +630,6 @@ __device__ __forceinline__ void row_tile(const StageArgs& a, long long L0, long 
     }
     pass_compute<C, T, N, E, 0>(v, t, tw2, 2);
     RowRest<C, T, N, E, 1, NP, 0>::run(v, srow, t, static_cast<const C*>(a.twr));
-    if constexpr (STAGE) stage_ending();
 
     if constexpr (OPR == 0) {
         row_sync<N / E>();
@@ -792,7 +785,6 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
     }
     pass_compute<C, T, N, E, 0>(v, t, tw, 1);
     RowRest<C, T, N, E, 1, NP, 0>::run(v, s + l * S::RP, t, static_cast<const C*>(a.twr));
-    if constexpr (N < 1024) stage_ending();  // longer tiles: costs more than it hides (1024^3: 4 us a stage)
     __syncthreads();  // the result tile overlaps other lines' exchange rows
     {
         const int u = PLast::out_u(t);
