@@ -323,9 +323,9 @@ p3_status p3_plan_set_z_hook(p3_plan plan, p3_z_hook fn, void* user);
  *     graph.  Results equal each plan's own within rounding (the power-of-two
  *     and plane-fused kernels a plan may use alone are not used here).
  *   Streams (nstreams >= 1): the plans' own launches spread over nstreams
- *     internal streams, or four if that is less and the grids average 3 M
- *     points or more (largest plans first, each to the least loaded
- *     stream), so the launches of different plans overlap on the GPU;
+ *     internal streams (largest plans first, each to the least loaded
+ *     stream; FP32 grids of 1.25 M points and more, and a few smaller ones
+ *     among many of these, to the least loaded of the first four), so the launches of different plans overlap on the GPU;
  *     results equal each plan's own bit for bit.
  *
  * p3_batch_create: plans (nplans >= 1, all created on the current device;

@@ -33,6 +33,7 @@ namespace p3 {
 p3_status run_direction(p3_plan plan, int dir, const void* in, void* out, void* ws, void* stream);
 size_t plan_workspace(p3_plan plan);
 double plan_work(p3_plan plan);
+bool plan_f32(p3_plan plan);
 int plan_device(p3_plan plan);
 p3_status generic_stages(p3_plan plan, int dir, std::vector<GenericStage>& out);
 p3_status check_generic_call(p3_plan plan, int dir, const void* in, void* out, void* ws);
@@ -211,16 +212,23 @@ p3_status p3_batch_create(p3_batch* out, int nplans, const p3_plan* plans, int n
         *out = b;
         return P3_OK;
     }
-    // Grids of 3 M points and more on average fill the SMs with a few of them in
-    // flight; more only push each other's arrays out of L2.  24 grids of 5.1 M
-    // points: 1.73 ms over 3 or 4 streams, 1.79 over 8, 1.88 over 16; 64 grids 4.62
-    // against 4.94 ms; eight of 25 M points the same over any number.  Smaller
-    // ones keep every stream (16 grids of 1.4 M: 378 us over 4, 340 over 16).
-    double work = 0.0;
-    for (int i = 0; i < nplans; ++i) work += p3::plan_work(plans[i]);
-    if (nstreams > 4 && work >= 3e6 * nplans) nstreams = 4;
     // longest-processing-time assignment: largest plans first, each to the
-    // stream with the least work so far
+    // stream with the least work so far.  FP32 grids of kLargePoints and more
+    // take turns on the first four streams: a few of them fill the SMs, and
+    // more at once push each other's arrays out of L2.  Forward + inverse of 16
+    // grids over 4 / 16 streams, replayed graph: 80^3 179 / 137 us, 100^3 201 /
+    // 189, 108^3 223 / 234, 120^3 296 / 331, 150^3 609 / 649; 24 grids of 48 to
+    // 384 points per side 1727 / 1786.  Smaller grids (and FP64 ones, which the
+    // arithmetic bounds: 16 of 160^3 2906 / 2646) keep every stream: 512^3 with
+    // forty 32^3 1382 us over four, 1126 when these run beside it.  A few small
+    // ones among many large ones queue with them instead: 64 grids of 48 to
+    // 384 points per side, a sixth of them small, 5359 us against 5610.
+    constexpr double kLargePoints = 1.25e6;
+    constexpr int kLargeStreams = 4;
+    int nlarge = 0, nsmall = 0;
+    for (int i = 0; i < nplans; ++i)
+        if (p3::plan_f32(plans[i])) ++(p3::plan_work(plans[i]) >= kLargePoints ? nlarge : nsmall);
+    const bool with_large = nlarge >= 2 * kLargeStreams && nlarge >= 2 * nsmall;
     std::vector<int> order((size_t)nplans);
     for (int i = 0; i < nplans; ++i) order[(size_t)i] = i;
     std::stable_sort(order.begin(), order.end(),
@@ -228,10 +236,14 @@ p3_status p3_batch_create(p3_batch* out, int nplans, const p3_plan* plans, int n
     std::vector<double> load((size_t)nstreams, 0.0);
     b->stream_of.assign((size_t)nplans, 0);
     for (int i : order) {
-        const int s = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+        const bool few = nstreams > kLargeStreams && p3::plan_f32(plans[i]) &&
+                         (with_large || p3::plan_work(plans[i]) >= kLargePoints);
+        const auto end = few ? load.begin() + kLargeStreams : load.end();
+        const int s = (int)(std::min_element(load.begin(), end) - load.begin());
         b->stream_of[(size_t)i] = s;
         load[(size_t)s] += p3::plan_work(plans[i]);
     }
+    nstreams = 1 + *std::max_element(b->stream_of.begin(), b->stream_of.end());  // those that got a plan
     b->streams.assign((size_t)nstreams, NULL);
     b->join.assign((size_t)nstreams, NULL);
     bool ok = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess;

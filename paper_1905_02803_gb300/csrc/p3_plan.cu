@@ -1632,6 +1632,7 @@ p3_status check_generic_call(p3_plan P, int dir, const void* in, void* out, void
     return check_call(P, dir, in, out, ws, P->st_unfused[dir]);
 }
 bool plan_batchable(p3_plan P) { return P && P->prec == P3_F32 && !P->hook; }
+bool plan_f32(p3_plan P) { return P && P->prec == P3_F32; }
 size_t plan_workspace(p3_plan plan) { return plan ? plan->ws_bytes : 0; }
 double plan_work(p3_plan plan) { return plan ? (double)plan->nx * plan->ny * plan->nz : 0.0; }
 int plan_device(p3_plan plan) { return plan ? plan->device : -1; }

@@ -196,3 +196,42 @@ def test_persistent_batch_rejects_fp64_and_stream_mode_counts_launches():
     b = Batch([p32, p64], nstreams=2)
     assert b.launches(0) == p32.launches(0) + p64.launches(0)
     assert P.p3_batch_wait_status(b.handle) == P.P3_OK
+
+
+# (grids, streams asked for, streams that the call's launches start on): a
+# large grid does not take the small ones' streams away; FP32 grids of 1.25 M
+# points and more share four, with a few smaller ones among eight or more of
+# them; FP64 grids, and other smaller ones, keep every stream
+ASSIGNED = [([(256, 256, 256)] + [(16, 16, 16)] * 4, "f32", 5, 5), ([(112, 112, 112)] * 6, "f32", 6, 4),
+            ([(104, 104, 104)] * 6, "f32", 6, 6), ([(112, 112, 112)] * 6, "f64", 6, 6),
+            ([(112, 112, 112)] * 2 + [(20, 20, 20)], "f32", 8, 3), ([(112, 112, 112)] * 8 + [(20, 20, 20)] * 4, "f32", 12, 4),
+            ([(112, 112, 112)] * 8 + [(20, 20, 20)] * 5, "f32", 13, 9)]
+
+
+@pytest.mark.parametrize("grids,prec,asked,used", ASSIGNED)
+def test_streams_of_a_batch(grids, prec, asked, used):
+    """A captured call has one first launch per internal stream in use."""
+    import ctypes
+
+    import torch
+    from paper_1905_02803_gb300.p3dfft import Batch, Plan
+    cu = ctypes.CDLL("libcuda.so.1")
+    plans = [Plan(*d, precision=prec) for d in grids]
+    xs = [p.empty_real().normal_() for p in plans]
+    Xs = [p.empty_complex() for p in plans]
+    b = Batch(plans, nstreams=asked)
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    graph, count = ctypes.c_void_p(), ctypes.c_size_t()
+    with torch.cuda.stream(s):
+        b.forward(xs, Xs)
+        torch.cuda.synchronize()
+        h = ctypes.c_void_p(s.cuda_stream)
+        assert cu.cuStreamBeginCapture_v2(h, 1) == 0  # thread-local mode
+        b.forward(xs, Xs)
+        assert cu.cuStreamEndCapture(h, ctypes.byref(graph)) == 0
+    assert cu.cuGraphGetNodes(graph, None, ctypes.byref(count)) == 0
+    assert count.value == sum(p.launches(0) for p in plans)
+    assert cu.cuGraphGetRootNodes(graph, None, ctypes.byref(count)) == 0
+    assert count.value == used
+    assert cu.cuGraphDestroy(graph) == 0
