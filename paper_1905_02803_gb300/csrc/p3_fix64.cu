@@ -100,6 +100,19 @@ bool fix64_configure(StageArgs& a, int shrink)
     return true;
 }
 
+const char* fix64_name(const StageArgs& a)
+{
+    // in the order of fx::Kind; forms 8, 10, 16
+#define P3_FX_NAMES(k) {"fix64_" k "_8", "fix64_" k "_10", "fix64_" k "_16"}
+    static const char* const names[][3] = {P3_FX_NAMES("cc"),  P3_FX_NAMES("cs"),  P3_FX_NAMES("sc"),  P3_FX_NAMES("ss"),
+                                           P3_FX_NAMES("ecc"), P3_FX_NAMES("ecs"), P3_FX_NAMES("esc"), P3_FX_NAMES("ess"),
+                                           P3_FX_NAMES("r2c"), P3_FX_NAMES("c2r"), P3_FX_NAMES("rp"),  P3_FX_NAMES("cp")};
+#undef P3_FX_NAMES
+    static_assert(sizeof(names) / sizeof(names[0]) == fx::K_CP + 1, "one row per kind");
+    const int cap = a.fix & 31;
+    return names[a.fix >> 5][cap == 8 ? 0 : cap == 10 ? 1 : 2];
+}
+
 cudaError_t fix64_prepare(const StageArgs& a)
 {
     return cudaFuncSetAttribute(pick(a.fix >> 5, a.fix & 31), cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024);

@@ -219,6 +219,8 @@ int fix64_threads(int n, int npass, const int* rad, int cap);
 // CTA that many times; false when none is left).
 bool fix64_configure(StageArgs& a, int shrink);
 cudaError_t fix64_prepare(const StageArgs& a);
+// "fix64_<kind>_<largest radix>" of a configured stage
+const char* fix64_name(const StageArgs& a);
 cudaError_t fix64_launch(const StageArgs& a, cudaStream_t s);
 // The inverse takes them at every size, the forward transform up to this many
 // points (Nx Ny Nz).  Their results are nearer to the exact transform than the

@@ -553,13 +553,7 @@ const char* op_name(int op)
 const char* kern_name(const StageArgs& a)
 {
     const int k = a.kern, tma = a.tma;
-    if (k == p3::KIND_FIX64) {
-        // power-of-two lengths keep the names of their FP32 counterparts
-        if (a.nfft < 64 || (a.nfft & (a.nfft - 1))) return "fix64";
-        if (a.op == p3::OP_R2C_HALF) return "pow2_row_r2c_fix64";
-        if (a.op == p3::OP_C2R_HALF) return "pow2_row_c2r_fix64";
-        return a.out_elem_fast ? "pow2_col_zyx_store_fix64" : a.in_elem_fast ? "pow2_col_zyx_load_fix64" : "pow2_col_fix64";
-    }
+    if (k == p3::KIND_FIX64) return p3::fix64_name(a);
     if (a.tc) return "tc_split_col";
     if (k == p3::KIND_LINE32) return tma ? "line32_bulk" : "line32";
     if (tma == 2) return "pow2_zrow_bulk";
@@ -1281,21 +1275,7 @@ p3_status p3_plan_create(p3_plan* out, int nx, int ny, int nz, p3_precision prec
                 continue;
             }
             std::string rs;
-            if (a.kern == p3::KIND_FIX64) {
-                // composite register butterflies as the native radices they are made of
-                for (int i = 0; i < a.npass; ++i) {
-                    switch (a.rad[i]) {
-                    case 6: rs += "2x3"; break;
-                    case 9: rs += "3x3"; break;
-                    case 10: rs += "2x5"; break;
-                    case 12: rs += "4x3"; break;
-                    case 14: rs += "2x7"; break;
-                    case 15: rs += "3x5"; break;
-                    default: rs += std::to_string(a.rad[i]); break;
-                    }
-                    if (i + 1 < a.npass) rs += "x";
-                }
-            } else if (a.kern != p3::KIND_GENERIC && a.kern != p3::KIND_LINE32) {
+            if (a.kern != p3::KIND_GENERIC && a.kern != p3::KIND_LINE32 && a.kern != p3::KIND_FIX64) {
                 // power-of-two kernels: radix E = nfft / tpl while it divides, then the rest
                 const int E = a.nfft / a.tpl;
                 int n = a.nfft;

@@ -153,6 +153,33 @@ def test_forms_against_oracle(shape, layout):
     assert ef <= 6e-16 and eb <= 6e-16, (ef, eb)
 
 
+# grid, Z transform, layout, then the kinds of the six stages in order
+NAMED = [((64, 128, 256), "fft", "zyx", "r2c cc cs sc cc c2r"), ((64, 54, 225), "fft", "xyz", "r2c cc cc cc cc c2r"),
+         ((15, 60, 90), "fft", "zyx", "rp cc cs sc cc cp"), ((30, 9, 65), "cheb", "zyx", "r2c cc ecs esc cc c2r"),
+         ((12, 36, 31), "sine", "xyz", "r2c cc ecc ecc cc c2r")]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape,z,layout,kinds", NAMED)
+def test_description_names_what_runs(shape, z, layout, kinds):
+    """The description gives each stage's own kernel and its passes: one radix
+    per pass (composite ones whole, none above the form's largest), whose
+    product is the line's length."""
+    from math import prod
+
+    from paper_1905_02803_gb300.p3dfft import Plan
+    desc = Plan(*shape, precision="f64", ttypes=("fft", "fft", z), layout=layout).describe()
+    lines = [dict(w.split("=", 1) for w in l.split() if "=" in w) for l in desc.splitlines() if "kernel=" in l]
+    assert len(lines) == 6
+    for f, kind in zip(lines, kinds.split()):
+        fix, got, form = f["kernel"].split("_")
+        assert (fix, got) == ("fix64", kind), f
+        rad = [int(r) for r in f["radices"].split("x")]
+        assert prod(rad) == int(f["nfft"]) and max(rad) <= int(form), f
+        if form != "16":  # one butterfly per thread: the narrowest pass sets the threads
+            assert int(f["tpl"]) == int(f["nfft"]) // min(rad), f
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("shape,ttypes", [((24, 20, 18), ("fft", "fft", "fft")), ((15, 9, 33), ("fft", "fft", "cheb")),
                                           ((64, 50, 31), ("fft", "fft", "sine"))])

@@ -64,7 +64,8 @@ def test_bluestein_lengths(shape, prec):
 
 # FP32 generic stages factor lengths with a factor 3, 5 or 7 into the fewest
 # passes over the native radices and the composite register butterflies 6,
-# 9, 10, 12, 14 and 15; FP64 stages keep the native radices.  Each composite
+# 9, 10, 12, 14 and 15; FP64 stages of this size run the fixed-point kernels,
+# which group the same radices by their own cost.  Each composite
 # appears in one of these plans (Y and Z lengths; X half-lengths of even Nx).
 COMPOSITE_CASES = [
     ((12, 54, 100), {"6", "9", "10"}),     # X 6; Y 54 = 9 x 6; Z 100 = 10 x 10
@@ -85,12 +86,11 @@ def test_composite_radices(shape, radices, layout):
                 used.update(w[len("radices="):].split("x"))
     assert radices <= used, (radices, used)
     assert ef <= TOL["f32"] and eb <= TOL["f32"], (ef, eb)
-    # the same grid in FP64 keeps the native radices 2, 3, 4, 5, 7, 8, 16
+    # the same grid in FP64
     ef64, eb64, plan64 = check_case(nx, ny, nz, "f64", layout=layout, seed=nx + nz)
     for line in plan64.describe().splitlines():
-        for w in line.split():
-            if w.startswith("radices="):
-                assert set(w[len("radices="):].split("x")) <= {"2", "3", "4", "5", "7", "8", "16"}, line
+        if "kernel=" in line:
+            assert "kernel=fix64_" in line, line
     assert ef64 <= TOL["f64"] and eb64 <= TOL["f64"], (ef64, eb64)
 
 
@@ -166,7 +166,8 @@ POW2_SHAPES = [(128, 64, 256), (256, 128, 64), (1024, 4, 6), (4096, 2, 3), (8192
 def test_pow2_kernels_parity(shape, prec, layout):
     nx, ny, nz = shape
     ef, eb, plan = check_case(nx, ny, nz, prec, layout=layout, seed=7)
-    assert "pow2_" in plan.describe()
+    # FP64: fixed point (longer volumes' double kernels: test_gpu_double.py)
+    assert ("pow2_" if prec == "f32" else "fix64_") in plan.describe()
     assert ef <= TOL[prec] and eb <= TOL[prec], (ef, eb)
 
 
@@ -175,7 +176,7 @@ def test_pow2_kernels_parity(shape, prec, layout):
 def test_pow2_chebyshev(nz, layout):
     for prec in ("f64", "f32"):
         ef, eb, plan = check_case(12, 6, nz, prec, ttypes=("fft", "fft", "cheb"), layout=layout, seed=nz)
-        assert "pow2_col" in plan.describe()
+        assert ("pow2_col" if prec == "f32" else "fix64_ec" if layout == "xyz" else "fix64_ecs") in plan.describe()
         assert ef <= TOL[prec] and eb <= TOL[prec], (prec, ef, eb)
 
 
@@ -196,15 +197,16 @@ def test_tc_split_parity(shape, layout):
 @pytest.mark.parametrize("layout", ["zyx", "xyz"])
 @pytest.mark.parametrize("prec", ["f64", "f32"])
 def test_sine_third_dimension(nz, layout, prec):
-    """DST-I in Z: odd extension to 2(Nz+1) points; Nz = 2^k - 1 runs the
-    power-of-two column kernels (sine variant), others the generic kernel
-    (Nz = 100: 202 = 2 * 101 is a Bluestein length)."""
+    """DST-I in Z: odd extension to 2(Nz+1) points; in FP32 Nz = 2^k - 1 runs
+    the power-of-two column kernels (sine variant), in FP64 the fixed-point
+    kernels (Nz = 100: 202 = 2 * 101 is a Bluestein length, on the generic
+    kernel in both)."""
     nx, ny = (24, 6) if nz >= 1023 else (34, 10)
     ef, eb, plan = check_case(nx, ny, nz, prec, ttypes=("fft", "fft", "sine"), layout=layout, seed=nz)
     assert ef <= TOL[prec] and eb <= TOL[prec], (ef, eb)
     assert "dst1" in plan.describe()
     if nz in (63, 127, 511, 1023, 2047):
-        assert "pow2_col" in plan.describe()
+        assert ("pow2_col" if prec == "f32" else "fix64_e") in plan.describe()
     assert plan.scale == nx * ny * 2 * (nz + 1)
 
 
