@@ -157,7 +157,7 @@ p3_status p3_plan_destroy(p3_plan plan);
  * Sect. 3.2).  in_real: Nx*Ny*Nz reals; out_cplx: H*Ny*Nz complex in the
  * plan's layout; workspace: p3_plan_workspace_bytes() bytes (may be NULL
  * when that is 0).  An infinity or a NaN in a line makes that line's transform
- * non-finite (FP64 fixed-point stages: NaN throughout).
+ * non-finite (in the FP64 fixed-point stages every output of it is NaN).
  * Errors: P3_ERR_INVALID (NULL plan/in/out, misaligned or
  * partly overlapping buffers), P3_ERR_UNSUPPORTED (in == out without
  * P3_FLAG_PADDED_REAL), P3_ERR_WORKSPACE,
@@ -209,15 +209,18 @@ p3_status p3_plan_describe(p3_plan plan, char* buf, size_t len);
 p3_status p3_plan_launches(p3_plan plan, int dir, int* launches);
 
 /*
- * The radix sequence a plan of precision prec gives the generic-kernel
- * stages of a line of n points (the Cooley-Tukey factorisation behind each
- * 1D FFT of Sect. 2; no device work, no GPU needed).  FP32 lengths with a
- * factor 3, 5 or 7 take the fewest passes over the native radices 2, 3, 4,
- * 5, 7, 8, 16 and the composite register butterflies up to 15; other
- * lengths take 16s first, then 8 / 4 / 2, then 3, 5, 7 (FP64 inverse
- * transforms, and forward ones of up to 12,582,912 points, run 64-bit fixed-point
- * kernels instead, which order and group these radices by their own cost).  radices receives
- * up to cap entries (the largest radix first), *npass their count.
+ * The radix sequence that the mixed-radix kernels in the arithmetic of
+ * precision prec take for a line of n points (the Cooley-Tukey factorisation
+ * behind each 1D FFT of Sect. 2; no device work, no GPU needed).  FP32 lengths
+ * with a factor 3, 5 or 7 take the fewest passes over the native radices 2, 3,
+ * 4, 5, 7, 8, 16 and the composite register butterflies up to 15; other
+ * lengths take 16s first, then 8 / 4 / 2, then 3, 5, 7.  FP64 plans use the
+ * sequence only where they run in double arithmetic: forward transforms of
+ * more than 12,582,912 points, and lines of more than 2304 points whose radices
+ * need more threads than a block of the 64-bit fixed-point kernels has (2430 or
+ * 3645).  Their other stages run these kernels, which order and group the
+ * radices by their own cost; p3_plan_describe() lists what a plan runs.  radices
+ * receives up to cap entries (the largest radix first), *npass their count.
  * P3_ERR_UNSUPPORTED when n has a prime factor above 7 (such lines run
  * Bluestein's algorithm over a power-of-two length) or the sequence is
  * longer than cap; P3_ERR_INVALID for n < 2, a bad precision or NULL

@@ -8,8 +8,8 @@
 // with one exponent per line (block floating point): a butterfly addition is
 // two 32-bit additions, a multiplication by a 64-bit twiddle part three
 // 32 x 32 -> 64 multiply-adds.  Doubles appear only in HBM.  Measured against
-// the double kernels: 32^3 forward + inverse 145 -> 31 us, 243 x 250 x 180 2450 ->
-// 764 us; inverse of 512^3 11.2 -> 3.1 ms (stages 3.45 / 3.45 / 4.27 -> 0.89 /
+// the double kernels: 32^3 forward + inverse 145 -> 30 us, 243 x 250 x 180 2450 ->
+// 767 us; inverse of 512^3 11.2 -> 3.1 ms (stages 3.45 / 3.45 / 4.27 -> 0.89 /
 // 0.87 / 1.33 ms), of the 480 x 360 x 257 channel grid 5.3 -> 1.4 ms.  What bounds
 // them now: issue slots 40-50 % busy, the rest waits for instruction fetch (long
 // unrolled passes), the double conversions and the dependent chains of 16 to 32
@@ -21,7 +21,10 @@
 // headroom (an OR over all magnitudes), so a pass loses only the bits that
 // the data really grew; twiddles carry 60 fractional bits and the butterfly
 // constants 64 (a double: 53).  The result is rounded once, to nearest, when
-// it becomes a double again.  Relative errors of a forward + inverse pair
+// it becomes a double again.  Components below 2^-5 of the line's largest keep
+// fewer bits than a double, those below 2^-58 none; as every output sums over
+// the whole line (over both rows of an odd pair), errors are relative to the
+// line's largest component, as they are in double arithmetic.  Relative errors of a forward + inverse pair
 // against a 64-bit reference: 3.5e-16 -> 2.7e-16 (32^3) and 6.0e-16 -> 3.7e-16
 // (243 x 250 x 180) from the double kernels to these.
 //

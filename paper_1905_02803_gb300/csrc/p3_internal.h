@@ -222,16 +222,24 @@ cudaError_t fix64_prepare(const StageArgs& a);
 // "fix64_<kind>_<largest radix>" of a configured stage
 const char* fix64_name(const StageArgs& a);
 cudaError_t fix64_launch(const StageArgs& a, cudaStream_t s);
-// The inverse takes them at every size, the forward transform up to this many
-// points (Nx Ny Nz).  Their results are nearer to the exact transform than the
-// double-arithmetic kernels' at every size, but they are other roundings: in
-// larger volumes the double kernels' own error in the spectrum's bins beside a
-// strong wave (up to 1.3e-12 of the typical bin at 512^3; 4.7e-13 once in fifty
-// runs at 250 x 256 x 250) exceeds the agreement with earlier results that
-// perf/cases.py holds outputs to (4.4e-13).  At 243 x 250 x 180 the largest of ten
-// runs was 2.4e-13.  The inverse's result is a field without such contrast:
-// at most 4.9e-15 at 512^3, 8.4e-15 on the 480 x 360 x 257 channel grid (six
-// runs each).
+// Lines that have a form (fixed_form in p3_plan.cu) take them in every inverse and
+// in forward transforms of up to this many points (Nx Ny Nz).  Neither accuracy
+// nor speed draws that line.  In fixed point a forward transform of 512^3 takes
+// 3.5 ms instead of 11.3, and its largest error against double-double arithmetic,
+// in the lines of the four strongest bins and three others of three fields of
+// waves and noise, is smaller at every size measured, as a multiple of the median
+// bin (double -> fixed point):
+//   512^3                        2.2e-12 .. 6.0e-12 -> 1.5e-12 .. 1.8e-12
+//   480 x 360 x 257, Chebyshev   7.1e-13 .. 2.2e-12 -> 3.8e-13 .. 4.7e-13
+//   250 x 256 x 250              6.5e-13 .. 7.4e-13 -> 3.4e-13 .. 6.7e-13
+//   256 x 256 x 196              6.9e-13 .. 2.4e-12 -> 3.1e-13 .. 7.4e-13
+// It keeps the spectra of larger volumes bit for bit what they were before these
+// kernels: the bins beside a strong wave carry the double kernels' own error, and
+// a spectrum rounded anew differs from an earlier one by as much.  Largest such
+// difference of a bin, as a multiple of the rms bin: 2.4e-13 in ten fields of
+// 243 x 250 x 180, 4.7e-13 in fifty of 250 x 256 x 250, 1.3e-12 at 512^3.  A field
+// has no such contrast, so an inverse differs from earlier ones by at most
+// 8.4e-15 of its rms (six runs at 512^3 and at 480 x 360 x 257).
 constexpr double kFix64MaxPoints = 12582912.0;
 
 // FP32 line kernels of smooth lengths (p3_line32.cu): configure a stage whose

@@ -1,6 +1,6 @@
 // Instantiations of the power-of-two stage kernels for double data: the forward
-// transform of large volumes (the inverse, and smaller volumes, run in fixed
-// point: p3_fix64.cuh).
+// transform of volumes of more than kFix64MaxPoints points (other stages of
+// these lengths run in fixed point: p3_fix64.cuh).
 #include "p3_pow2.cuh"
 
 namespace p3 {

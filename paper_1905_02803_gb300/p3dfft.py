@@ -272,8 +272,9 @@ def p3_plan_describe(plan) -> str:
 
 
 def p3_plan_factor(n: int, precision: str = "f32"):
-    """Radix sequence of the generic-kernel stages of an n-point line (no GPU
-    needed); None when n has a prime factor above 7."""
+    """Radix sequence of an n-point line in the mixed-radix kernels of that
+    precision's own arithmetic (FP64 stages in fixed point choose their own: see
+    Plan.describe); no GPU needed.  None when n has a prime factor above 7."""
     prec = {"f32": P3_F32, "f64": P3_F64}[precision]
     buf = (ctypes.c_int * 32)()
     cnt = ctypes.c_int()

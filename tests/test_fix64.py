@@ -264,10 +264,87 @@ def test_lines_of_the_smallest_denormals(shape, z, layout):
     assert (back - wantb).abs().max().item() <= boundb < 0.2 * wantb.abs().max().item()
 
 
+# a line whose passes need more threads than a block has (radix 9 of 2430: 270)
+# has no fixed-point form: double arithmetic in both directions
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", [(4860, 2, 3), (2835, 3, 5), (6, 3645, 4), (3, 4, 2916), (5, 2430, 2), (2, 3, 4050)])
+@pytest.mark.parametrize("layout", ["zyx", "xyz"])
+def test_lengths_without_a_form(shape, layout):
+    from _gpu_helpers import check_case
+    ef, eb, plan = check_case(*shape, "f64", layout=layout, seed=sum(shape))
+    long = [l for l in plan.describe().splitlines() if "kernel=" in l and int(l.split("nfft=")[1].split()[0]) > 2304]
+    assert len(long) == 2 and all("kernel=generic" in l for l in long), long
+    # half a unit of the last place per butterfly level (12 of them here, and 4
+    # in the short lines)
+    assert ef <= 18e-16 and eb <= 18e-16, (ef, eb)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", [(96, 64, 60), (75, 50, 81)])
+@pytest.mark.parametrize("layout", ["zyx", "xyz"])
+def test_steep_spectrum(shape, layout):
+    """Amplitudes that fall by 30 orders of magnitude over the bins.  A line has
+    one exponent, so its error is relative to its largest value, as a sum over
+    the line in double arithmetic is to the largest term: both directions
+    are as near to the oracle as for a flat spectrum, and no single bin is
+    further off than that error would be if it all fell on one of them."""
+    import numpy as np
+    import torch
+
+    import oracle as O
+    from _gpu_helpers import random_complex, rel_l2
+    from paper_1905_02803_gb300.p3dfft import Plan
+    nx, ny, nz = shape
+    kz, ky, kx = (np.minimum(np.arange(n), n - np.arange(n)) / (n / 2) for n in (nz, ny, nx))
+    k = kz[:, None, None] + ky[None, :, None] + kx[None, None, :nx // 2 + 1]
+    F = random_complex(k.shape, 5) * 10.0 ** (-10 * k)
+    plan = Plan(nx, ny, nz, precision="f64", layout=layout)
+    y = plan.backward(torch.from_numpy(O.to_zyx(F) if layout == "zyx" else F).cuda()).cpu().numpy()
+    ref = O.backward(F, nx)
+    assert rel_l2(y, ref) <= 6e-16
+    X = plan.forward(torch.from_numpy(ref).cuda()).cpu().numpy()
+    X = O.from_zyx(X) if layout == "zyx" else X
+    Xr = O.forward(ref)
+    assert rel_l2(X, Xr) <= 6e-16
+    assert np.abs(X - Xr).max() <= 6e-16 * np.linalg.norm(Xr.ravel())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nx", [96, 75])
+@pytest.mark.parametrize("layout", ["zyx", "xyz"])
+def test_rows_of_unlike_size(nx, layout):
+    """Rows alone (no Y or Z transform), every other one 1e-9 of its
+    neighbour.  Even rows are as accurate each for itself; odd ones run two to a
+    complex line, in double arithmetic as here, so their errors are relative to
+    the pair."""
+    import numpy as np
+    import torch
+
+    import oracle as O
+    from _gpu_helpers import random_complex
+    from paper_1905_02803_gb300 import inputs
+    from paper_1905_02803_gb300.p3dfft import Plan
+    ny, nz = 8, 6
+    tt = (O.FFT, O.EMPTY, O.EMPTY)
+    size = np.where(np.arange(ny) % 2 == 0, 1.0, 1e-9)[None, :, None]
+    f = inputs.uniform_field((nz, ny, nx), 9) * size
+    F = random_complex((nz, ny, nx // 2 + 1), 4) * size
+    plan = Plan(nx, ny, nz, precision="f64", ttypes=("fft", "empty", "empty"), layout=layout)
+    X = plan.forward(torch.from_numpy(f).cuda()).cpu().numpy()
+    X = O.from_zyx(X) if layout == "zyx" else X
+    y = plan.backward(torch.from_numpy(O.to_zyx(F) if layout == "zyx" else F).cuda()).cpu().numpy()
+    for got, ref in ((X, O.forward(f, tt)), (y, O.backward(F, nx, tt))):
+        err, norm = np.linalg.norm(got - ref, axis=2), np.linalg.norm(ref, axis=2)
+        if nx % 2:
+            norm[:, 1::2] = norm[:, ::2]
+        assert (err <= 6e-16 * norm).all(), (err / norm).max()
+
+
 @pytest.mark.gpu
 def test_volume_limit_keeps_double_kernels():
     """Forward transforms of more than 12,582,912 points keep the double
-    kernels; every inverse runs in fixed point."""
+    kernels (test_gpu_double.py runs them); every inverse of a length with a form
+    runs in fixed point."""
     from paper_1905_02803_gb300.p3dfft import Plan
     for nz, fixed in ((192, True), (196, False)):
         lines = [w for w in Plan(256, 256, nz, precision="f64").describe().splitlines() if "kernel=" in w]
