@@ -1,5 +1,7 @@
-// Tiles that arrive in shared memory by tensor or bulk copies: the barrier that
-// counts their bytes and the bounded wait for it.
+// What the stage kernels share in moving tiles: line bases, the walk over a
+// tile's values, 8- and 16-byte copies into shared memory, and, for tiles that
+// arrive by tensor or bulk copies, the barrier that counts their bytes and the
+// bounded wait for it.
 #pragma once
 
 #include "p3_internal.h"
@@ -7,6 +9,47 @@
 namespace p3 {
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+// Offset (elements) of line L.
+__device__ __forceinline__ long long line_base(const LineMap& m, long long L)
+{
+    if (m.pm) {  // L < 2^31: quotient by multiply-high (line_magic)
+        const unsigned u = (unsigned)L;
+        const unsigned q = (unsigned)(((unsigned long long)u * m.pm) >> m.ps);
+        const unsigned r = u - q * (unsigned)m.per;
+        return (long long)q * m.gstride + (long long)r * m.lstride;
+    }
+    return (L / m.per) * m.gstride + (L % m.per) * m.lstride;
+}
+
+// Calls f(l, e) for every value of a tile of `rows` lines of `len` values,
+// threads walking the values together; the loop unrolled UNROLL times.
+template <int UNROLL, class F> __device__ __forceinline__ void walk(int rows, int len, F f)
+{
+    const int NT = blockDim.x, tid = threadIdx.x;
+    int l = tid / len, e = tid - l * len;
+    const int dq = NT / len, dr = NT - dq * len;
+#pragma unroll UNROLL
+    while (l < rows) {
+        f(l, e);
+        e += dr;
+        l += dq;
+        if (e >= len) {
+            e -= len;
+            ++l;
+        }
+    }
+}
+
+__device__ __forceinline__ void cp_async16(unsigned d, const void* g)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(g) : "memory");
+}
+__device__ __forceinline__ void cp_async8(unsigned d, const void* g)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(g) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 __device__ __forceinline__ bool mbar_try_wait(unsigned bar, unsigned parity)
 {

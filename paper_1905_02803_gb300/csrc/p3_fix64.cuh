@@ -42,6 +42,7 @@
 
 #include <cuda_runtime.h>
 
+#include "p3_copy.cuh"
 #include "p3_internal.h"
 #include "p3_launch.cuh"
 
@@ -449,28 +450,6 @@ struct Shared {
     int odd[kMaxB];                           // f is not 1
 };
 
-__device__ __forceinline__ ll base_of(const LineMap& m, ll L)
-{
-    if (m.pm) {
-        const unsigned u = (unsigned)L;
-        const unsigned q = (unsigned)(((unsigned long long)u * m.pm) >> m.ps);
-        const unsigned r = u - q * (unsigned)m.per;
-        return (ll)q * m.gstride + (ll)r * m.lstride;
-    }
-    return (L / m.per) * m.gstride + (L % m.per) * m.lstride;
-}
-
-__device__ __forceinline__ void cp16(const void* d, const void* g)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(d)), "l"(g)
-                 : "memory");
-}
-__device__ __forceinline__ void cp8(const void* d, const void* g)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(d)), "l"(g)
-                 : "memory");
-}
-
 // Combines a per-thread word over the lanes of a warp that share a line and
 // posts it to the line's word (B a power of two; every lane takes part).
 template <bool MAXOP> __device__ __forceinline__ void post(unsigned m, unsigned* w, int B, int l)
@@ -835,24 +814,6 @@ __device__ __forceinline__ void pass_any(const StageArgs& a, Q* s, Shared& sh, T
     }
 }
 
-// Calls f(l, e) for every value of a tile of `rows` lines of `len` values,
-// threads walking the values together.
-template <class F> __device__ __forceinline__ void walk(int rows, int len, F f)
-{
-    const int NT = blockDim.x, tid = threadIdx.x;
-    int l = tid / len, e = tid - l * len;
-    const int dq = NT / len, dr = NT - dq * len;
-    while (l < rows) {
-        f(l, e);
-        e += dr;
-        l += dq;
-        if (e >= len) {
-            e -= len;
-            ++l;
-        }
-    }
-}
-
 template <int K, int CAP>
 __global__ void __launch_bounds__(kThreads, CAP <= 10 ? 4 : 2) kernel(const __grid_constant__ StageArgs a)
 {
@@ -871,16 +832,16 @@ __global__ void __launch_bounds__(kThreads, CAP <= 10 ? 4 : 2) kernel(const __gr
         if (tid < rows) {
             has = 1;
             if (K == K_RP || K == K_CP) {
-                bi = base_of(a.in, 2 * L);
-                bo = base_of(a.out, 2 * L);
+                bi = line_base(a.in, 2 * L);
+                bo = line_base(a.out, 2 * L);
                 if (2 * L + 1 < a.nrows) {
                     has = 2;
-                    bi2 = base_of(a.in, 2 * L + 1);
-                    bo2 = base_of(a.out, 2 * L + 1);
+                    bi2 = line_base(a.in, 2 * L + 1);
+                    bo2 = line_base(a.out, 2 * L + 1);
                 }
             } else {
-                bi = base_of(a.in, L);
-                bo = base_of(a.out, L);
+                bi = line_base(a.in, L);
+                bo = line_base(a.out, L);
             }
         }
         sh.has[tid] = has;
@@ -895,29 +856,29 @@ __global__ void __launch_bounds__(kThreads, CAP <= 10 ? 4 : 2) kernel(const __gr
     if constexpr (in_staged<K>()) {
         if constexpr (K == K_RP) {
             const double* f = static_cast<const double*>(a.src);
-            walk(rows, n, [&](int l, int e) {
+            walk<1>(rows, n, [&](int l, int e) {
                 double* d = reinterpret_cast<double*>(s + e * LDB + l);
-                cp8(d, f + sh.bin[l] + e);
-                if (sh.has[l] == 2) cp8(d + 1, f + sh.bin2[l] + e);
+                cp_async8(smem_u32(d), f + sh.bin[l] + e);
+                if (sh.has[l] == 2) cp_async8(smem_u32(d + 1), f + sh.bin2[l] + e);
                 else d[1] = 0.0;
             });
         } else if constexpr (K == K_CP) {
             const double2* F = static_cast<const double2*>(a.src);
             const int H = a.n_in;
-            walk(rows, H, [&](int l, int e) {
-                cp16(s + e * LDB + l, F + sh.bin[l] + e);
+            walk<1>(rows, H, [&](int l, int e) {
+                cp_async16(smem_u32(s + e * LDB + l), F + sh.bin[l] + e);
                 Q* d = s + (H + e) * LDB + l;
-                if (sh.has[l] == 2) cp16(d, F + sh.bin2[l] + e);
+                if (sh.has[l] == 2) cp_async16(smem_u32(d), F + sh.bin2[l] + e);
                 else *d = Q{0, 0};
             });
         } else if constexpr (K == K_R2C) {
             const double* f = static_cast<const double*>(a.src);
-            walk(rows, n, [&](int l, int e) { cp16(s + e * LDB + l, f + sh.bin[l] + 2 * e); });
+            walk<1>(rows, n, [&](int l, int e) { cp_async16(smem_u32(s + e * LDB + l), f + sh.bin[l] + 2 * e); });
         } else {  // contiguous complex lines; C2R: n + 1 bins
             const double2* F = static_cast<const double2*>(a.src);
-            walk(rows, K == K_C2R ? n + 1 : a.n_in, [&](int l, int e) { cp16(s + e * LDB + l, F + sh.bin[l] + e); });
+            walk<1>(rows, K == K_C2R ? n + 1 : a.n_in, [&](int l, int e) { cp_async16(smem_u32(s + e * LDB + l), F + sh.bin[l] + e); });
         }
-        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        cp_async_wait();
         __syncthreads();
     }
 
@@ -945,17 +906,17 @@ __global__ void __launch_bounds__(kThreads, CAP <= 10 ? 4 : 2) kernel(const __gr
         if constexpr (K == K_CS || K == K_SS) {
             double2* F = static_cast<double2*>(a.dst);
             const bool inv = a.sign > 0;  // the inverse-sign bin k is the forward bin -k
-            walk(rows, n, [&](int l, int e) { F[sh.bout[l] + e] = out(s[(inv && e > 0 ? n - e : e) * LDB + l], l); });
+            walk<1>(rows, n, [&](int l, int e) { F[sh.bout[l] + e] = out(s[(inv && e > 0 ? n - e : e) * LDB + l], l); });
         } else if constexpr (K == K_ECS || K == K_ESS) {
             double2* F = static_cast<double2*>(a.dst);
             const bool dst1 = a.op == OP_DST1;  // i times bin e + 1
-            walk(rows, a.n_out, [&](int l, int e) {
+            walk<1>(rows, a.n_out, [&](int l, int e) {
                 const double2 d = out(s[(e + (dst1 ? 1 : 0)) * LDB + l], l);
                 F[sh.bout[l] + e] = dst1 ? make_double2(-d.y, d.x) : d;
             });
         } else if constexpr (K == K_C2R) {
             double* f = static_cast<double*>(a.dst);
-            walk(rows, n, [&](int l, int e) {
+            walk<1>(rows, n, [&](int l, int e) {
                 const double2 d = out(s[e * LDB + l], l);
                 *reinterpret_cast<double2*>(f + sh.bout[l] + 2 * e) = make_double2(d.y, d.x);
             });
@@ -965,7 +926,7 @@ __global__ void __launch_bounds__(kThreads, CAP <= 10 ? 4 : 2) kernel(const __gr
             // sums stay below 2^62.5 (the last pass left room for them)
             double2* F = static_cast<double2*>(a.dst);
             const int4* w2 = static_cast<const int4*>(a.tw2);
-            walk(rows, n / 2 + 1, [&](int l, int k) {
+            walk<1>(rows, n / 2 + 1, [&](int l, int k) {
                 const Q zk = s[k * LDB + l];
                 Q zm = s[(k == 0 ? 0 : n - k) * LDB + l];
                 zm.y = -zm.y;
@@ -978,7 +939,7 @@ __global__ void __launch_bounds__(kThreads, CAP <= 10 ? 4 : 2) kernel(const __gr
         } else if constexpr (K == K_RP) {
             // X1[k] = (Z[k] + conj Z[n-k]) / 2, X2[k] = -i (Z[k] - conj Z[n-k]) / 2
             double2* F = static_cast<double2*>(a.dst);
-            walk(rows, a.n_out, [&](int l, int k) {
+            walk<1>(rows, a.n_out, [&](int l, int k) {
                 Q zk = s[k * LDB + l], zm = s[(k == 0 ? 0 : n - k) * LDB + l];
                 zk = Q{zk.x >> 1, zk.y >> 1};
                 zm = Q{zm.x >> 1, zm.y >> 1};
@@ -987,7 +948,7 @@ __global__ void __launch_bounds__(kThreads, CAP <= 10 ? 4 : 2) kernel(const __gr
             });
         } else {  // K_CP: real rows from the (swapped) result
             double* f = static_cast<double*>(a.dst);
-            walk(rows, a.n_out, [&](int l, int e) {
+            walk<1>(rows, a.n_out, [&](int l, int e) {
                 const double2 d = out(s[e * LDB + l], l);
                 f[sh.bout[l] + e] = d.y;
                 if (sh.has[l] == 2) f[sh.bout2[l] + e] = d.x;

@@ -16,6 +16,7 @@
 // sequence between pencils.
 #include <cstddef>
 
+#include "p3_copy.cuh"
 #include "p3_dft.cuh"
 #include "p3_internal.h"
 #include "p3_launch.cuh"
@@ -132,17 +133,6 @@ __device__ __forceinline__ C* run_passes(C* buf0, C* buf1, int LDB, int l, int t
         dst = tmp;
     }
     return src;
-}
-
-__device__ __forceinline__ long long line_base(const LineMap& m, long long L)
-{
-    if (m.pm) {  // L < 2^31: quotient by multiply-high (line_magic)
-        const unsigned u = (unsigned)L;
-        const unsigned q = (unsigned)(((unsigned long long)u * m.pm) >> m.ps);
-        const unsigned r = u - q * (unsigned)m.per;
-        return (long long)q * m.gstride + (long long)r * m.lstride;
-    }
-    return (L / m.per) * m.gstride + (L % m.per) * m.lstride;
 }
 
 // Value placed in shared-memory slot e of a line before the FFT (the op
@@ -377,15 +367,8 @@ __device__ __forceinline__ const C* direct_src(const StageArgs& a, long long bas
 template <class C>
 __device__ __forceinline__ void copy_async(unsigned d, const C* src)
 {
-    if constexpr (sizeof(C) == 16)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
-}
-
-__device__ __forceinline__ void copy_async_wait()
-{
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    if constexpr (sizeof(C) == 16) cp_async16(d, src);
+    else cp_async8(d, src);
 }
 
 // Writes output elements e0, e0 + de, ... (< n_out) of one line, whose
@@ -535,7 +518,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, long long tile, u
                     copy_async((unsigned)__cvta_generic_to_shared(s1 + l), direct_src<C, T>(a, base, nload));
             }
         }
-        copy_async_wait();
+        cp_async_wait();
         if (sw_in && a.npass == 0) {
             for (int l = l0; l < B; l += dl) {
                 if (L0 + l >= a.nlines) break;

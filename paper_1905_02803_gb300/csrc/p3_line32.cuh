@@ -70,23 +70,6 @@ struct Shared {
     ll bin[kMaxB], bout[kMaxB];  // line bases (elements)
 };
 
-__device__ __forceinline__ ll base_of(const LineMap& m, ll L)
-{
-    if (m.pm) {
-        const unsigned u = (unsigned)L;
-        const unsigned q = (unsigned)(((unsigned long long)u * m.pm) >> m.ps);
-        const unsigned r = u - q * (unsigned)m.per;
-        return (ll)q * m.gstride + (ll)r * m.lstride;
-    }
-    return (L / m.per) * m.gstride + (L % m.per) * m.lstride;
-}
-
-__device__ __forceinline__ void cp_async8(const void* d, const void* g)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(d)), "l"(g)
-                 : "memory");
-}
-
 // Butterflies past the end (and threads and lines past theirs) read the last
 // one's values, which exist, and write nothing.
 __device__ __forceinline__ int clamp(int j, int nb) { return j < nb ? j : nb - 1; }
@@ -266,25 +249,6 @@ __device__ __forceinline__ void pass_any(const StageArgs& a, C* s, const Shared&
     }
 }
 
-// Calls f(l, e) for every value of a tile of `rows` lines of `len` values,
-// threads walking the values together.
-template <class F> __device__ __forceinline__ void walk(int rows, int len, F f)
-{
-    const int NT = blockDim.x, tid = threadIdx.x;
-    int l = tid / len, e = tid - l * len;
-    const int dq = NT / len, dr = NT - dq * len;
-#pragma unroll 4
-    while (l < rows) {
-        f(l, e);
-        e += dr;
-        l += dq;
-        if (e >= len) {
-            e -= len;
-            ++l;
-        }
-    }
-}
-
 template <int K, bool BULK = false>
 __global__ void __launch_bounds__(kThreadsMost, 2) kernel(const __grid_constant__ StageArgs a)
 {
@@ -302,8 +266,8 @@ __global__ void __launch_bounds__(kThreadsMost, 2) kernel(const __grid_constant_
     const int rows = (int)(a.nlines - L0 < B ? a.nlines - L0 : B);
     if (tid < B) {
         const ll L = tid < rows ? L0 + tid : L0;  // lines past the end read the tile's first
-        sh.bin[tid] = base_of(a.in, L);
-        sh.bout[tid] = base_of(a.out, L);
+        sh.bin[tid] = line_base(a.in, L);
+        sh.bout[tid] = line_base(a.out, L);
     }
     __syncthreads();
     stage_begin();
@@ -317,8 +281,8 @@ __global__ void __launch_bounds__(kThreadsMost, 2) kernel(const __grid_constant_
         if (!copy_bar_wait(a, bar)) return;
     } else if constexpr (in_staged<K>()) {
         const C* F = static_cast<const C*>(a.src);
-        walk(rows, a.n_in, [&](int l, int e) { cp_async8(s + e * LDB + l, F + sh.bin[l] + e); });
-        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        walk<4>(rows, a.n_in, [&](int l, int e) { cp_async8(smem_u32(s + e * LDB + l), F + sh.bin[l] + e); });
+        cp_async_wait();
         __syncthreads();
     }
 
@@ -339,17 +303,17 @@ __global__ void __launch_bounds__(kThreadsMost, 2) kernel(const __grid_constant_
         C* F = static_cast<C*>(a.dst);
         if (n % 2 == 0 && a.out.lstride % 2 == 0 && a.out.gstride % 2 == 0) {
             // lines start on 16 bytes: two values per store
-            walk(rows, n / 2, [&](int l, int h) {
+            walk<4>(rows, n / 2, [&](int l, int h) {
                 const C x = s[2 * h * LDB + l], y = s[(2 * h + 1) * LDB + l];
                 *reinterpret_cast<float4*>(F + sh.bout[l] + 2 * h) = make_float4(x.x, x.y, y.x, y.y);
             });
         } else {
-            walk(rows, n, [&](int l, int e) { F[sh.bout[l] + e] = s[e * LDB + l]; });
+            walk<4>(rows, n, [&](int l, int e) { F[sh.bout[l] + e] = s[e * LDB + l]; });
         }
     } else if constexpr (K == K_ECS) {
         C* F = static_cast<C*>(a.dst);
         const bool dst1 = a.op == OP_DST1;  // i times bin e + 1
-        walk(rows, a.n_out, [&](int l, int e) {
+        walk<4>(rows, a.n_out, [&](int l, int e) {
             const C x = s[(e + (dst1 ? 1 : 0)) * LDB + l];
             F[sh.bout[l] + e] = dst1 ? mk<C>(-x.y, x.x) : x;
         });
@@ -528,14 +492,14 @@ template <int K> __global__ void __launch_bounds__(kThreadsMost, 2) row_kernel(c
     ll L = (ll)blockIdx.x * B + l;
     th.valid = in && L < a.nlines;
     if (L >= a.nlines) L = a.nlines - 1;
-    th.bi = base_of(a.in, PAIR ? 2 * L : L);
-    th.bo = base_of(a.out, PAIR ? 2 * L : L);
+    th.bi = line_base(a.in, PAIR ? 2 * L : L);
+    th.bo = line_base(a.out, PAIR ? 2 * L : L);
     th.bi2 = th.bi;
     th.bo2 = th.bo;
     th.two = PAIR && 2 * L + 1 < a.nrows;
     if (th.two) {
-        th.bi2 = base_of(a.in, 2 * L + 1);
-        th.bo2 = base_of(a.out, 2 * L + 1);
+        th.bi2 = line_base(a.in, 2 * L + 1);
+        th.bo2 = line_base(a.out, 2 * L + 1);
     }
     const int ps = a.LDB;
     C* sl = s + l * rpitch(n, ps);

@@ -101,17 +101,6 @@ template <int NT, int CSIZE, int E> struct MinBlocks {
         CSIZE == 8 ? (E == 32 ? (NT >= 512 ? 1 : P3_E32_MINB) : (NT >= 512 ? 2 : 3)) : (NT >= 512 ? 1 : 2);
 };
 
-__device__ __forceinline__ long long lbase(const LineMap& m, long long L)
-{
-    if (m.pm) {  // L < 2^31: quotient by multiply-high (line_magic)
-        const unsigned u = (unsigned)L;
-        const unsigned q = (unsigned)(((unsigned long long)u * m.pm) >> m.ps);
-        const unsigned r = u - q * (unsigned)m.per;
-        return (long long)q * m.gstride + (long long)r * m.lstride;
-    }
-    return (L / m.per) * m.gstride + (L % m.per) * m.lstride;
-}
-
 // Line of lane l of tile `tile` (tile i takes lines i * B + l); false past
 // the end.
 __device__ __forceinline__ bool tile_line(const StageArgs& a, int B, long long tile, int l, long long* L)
@@ -263,7 +252,7 @@ __device__ __forceinline__ void col_tile(const StageArgs& a, long long tile, lon
     typedef PassIdx<N, E, 0> P0;
 
     if constexpr (MODE != 2) {
-        const C* src = static_cast<const C*>(a.src) + off + (valid ? lbase(a.in, L) : 0);
+        const C* src = static_cast<const C*>(a.src) + off + (valid ? line_base(a.in, L) : 0);
         const long long es = a.in.es;
 #pragma unroll
         for (int b = 0; b < P0::BM; ++b)
@@ -287,7 +276,7 @@ __device__ __forceinline__ void col_tile(const StageArgs& a, long long tile, lon
         const int le = Ef::line(tid);
         long long Le;
         const bool ve = tile_line(a, B, tile, le, &Le);
-        const C* src = static_cast<const C*>(a.src) + off + (ve ? lbase(a.in, Le) : 0);
+        const C* src = static_cast<const C*>(a.src) + off + (ve ? line_base(a.in, Le) : 0);
         if constexpr (DST) {
             for (int c = Ef::chunk0(tid); c < N; c += Ef::STEP) {
                 C x = (ve && c != 0 && c != M) ? ldx<LP>(src + (c < M ? c - 1 : N - 1 - c)) : zero;
@@ -321,7 +310,7 @@ __device__ __forceinline__ void col_tile(const StageArgs& a, long long tile, lon
     typedef PassIdx<N, E, NP - 1> PLast;
     if constexpr (MODE != 1) {
         if (valid) {
-            C* dst = static_cast<C*>(a.dst) + off + lbase(a.out, L);
+            C* dst = static_cast<C*>(a.dst) + off + line_base(a.out, L);
             const long long es = a.out.es;
             const int u = PLast::out_u(t);
 #pragma unroll
@@ -351,7 +340,7 @@ __device__ __forceinline__ void col_tile(const StageArgs& a, long long tile, lon
         const int le = Ef::line(tid);
         long long Le;
         if (tile_line(a, B, tile, le, &Le)) {
-            C* dst = static_cast<C*>(a.dst) + off + lbase(a.out, Le);
+            C* dst = static_cast<C*>(a.dst) + off + line_base(a.out, Le);
             if constexpr (DST) {
                 for (int c = Ef::chunk0(tid); c < M - 1; c += Ef::STEP) {
                     const C x = s[S::at(c + 1, le)];
@@ -471,7 +460,7 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
     typedef PassIdx<N, E, NP - 1> PLast;
     if constexpr (!ZYX) {
         if (L0 + l < a.nlines) {
-            C* dst = static_cast<C*>(a.dst) + lbase(a.out, L0 + l);
+            C* dst = static_cast<C*>(a.dst) + line_base(a.out, L0 + l);
             const long long es = a.out.es;
             const int u = PLast::out_u(t);
 #pragma unroll
@@ -501,7 +490,7 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
     const int le = Ef::line(tid);
     const long long Le = L0 + le;
     if (Le < a.nlines) {
-        C* dst = static_cast<C*>(a.dst) + lbase(a.out, Le);
+        C* dst = static_cast<C*>(a.dst) + line_base(a.out, Le);
         if constexpr (DST) {
             for (int c = Ef::chunk0(tid); c < M - 1; c += Ef::STEP) {
                 const C x = s[S::at(c + 1, le)];
@@ -754,7 +743,7 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
                              smem_u32(s)),
-                         "l"(static_cast<const C*>(a.src) + lbase(a.in, L0)), "r"(bytes), "r"(bar)
+                         "l"(static_cast<const C*>(a.src) + line_base(a.in, L0)), "r"(bytes), "r"(bar)
                          : "memory");
         }
         if (!copy_bar_wait(a, bar)) return;
@@ -767,7 +756,7 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
             }
         __syncthreads();  // the exchange rows overlap the bulk tile
     } else {
-        const C* src = static_cast<const C*>(a.src) + (valid ? lbase(a.in, L) : 0);
+        const C* src = static_cast<const C*>(a.src) + (valid ? line_base(a.in, L) : 0);
 #pragma unroll
         for (int b = 0; b < P0::BM; ++b)
 #pragma unroll
@@ -801,7 +790,7 @@ __global__ void __launch_bounds__(B * (N / E), (MinBlocks<B * (N / E), 2 * sizeo
     const int ll = tid % B;
     const long long LL = L0 + ll;
     if (LL < a.nlines) {
-        C* dst = static_cast<C*>(a.dst) + lbase(a.out, LL);
+        C* dst = static_cast<C*>(a.dst) + line_base(a.out, LL);
         const long long es = a.out.es;
         for (int c = tid / B; c < NOUT; c += NT / B) {
             const int e = DST ? c + 1 : c;

@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(NT, 1) col_tc_kernel(const __grid_constant__ S
         const long long Lg = (long long)blockIdx.x * B + g;  // this lane's line in the B operand
         const bool vg = Lg < a.nlines;
         if constexpr (MODE != 2) {
-            const C* src = static_cast<const C*>(a.src) + (vg ? lbase(a.in, Lg) : 0);
+            const C* src = static_cast<const C*>(a.src) + (vg ? line_base(a.in, Lg) : 0);
             const long long es = a.in.es;
 #pragma unroll
             for (int n = 0; n < 4; ++n)
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(NT, 1) col_tc_kernel(const __grid_constant__ S
             const int le = Ef::line(tid);
             long long Le = (long long)blockIdx.x * B + le;
             const bool ve = Le < a.nlines;
-            const C* src = static_cast<const C*>(a.src) + (ve ? lbase(a.in, Le) : 0);
+            const C* src = static_cast<const C*>(a.src) + (ve ? line_base(a.in, Le) : 0);
             const float4* src4 = reinterpret_cast<const float4*>(src);
             for (int c = Ef::chunk0(tid); c < N / 2; c += Ef::STEP) {
                 float4 v = ve ? src4[c] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(NT, 1) col_tc_kernel(const __grid_constant__ S
     }
     if constexpr (MODE != 1) {
         if (valid) {
-            C* dst = static_cast<C*>(a.dst) + lbase(a.out, L);
+            C* dst = static_cast<C*>(a.dst) + line_base(a.out, L);
             const long long es = a.out.es;
 #pragma unroll
             for (int b = 0; b < 4; ++b)
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(NT, 1) col_tc_kernel(const __grid_constant__ S
         const int le = Ef::line(tid);
         const long long Le = (long long)blockIdx.x * B + le;
         if (Le < a.nlines) {
-            C* dst = static_cast<C*>(a.dst) + lbase(a.out, Le);
+            C* dst = static_cast<C*>(a.dst) + line_base(a.out, Le);
             float4* dst4 = reinterpret_cast<float4*>(dst);
             for (int c = Ef::chunk0(tid); c < N / 2; c += Ef::STEP) {
                 C x0 = s[S::at(2 * c, le)], x1 = s[S::at(2 * c + 1, le)];
