@@ -679,10 +679,11 @@ def _report_one(name, dims, prec, ttypes, layout, kind, mode="", *, steps, warmu
            "ms": round(ms, 4), "gflops": round(gflops, 1), "stage_model_bytes": pair_bytes,
            "hbm_roofline_ms": round(roof_ms, 4), "hbm_roofline_frac": round(roof_ms / ms, 4)}
     if prec == "f64":
-        # the FP64 transforms are bound by the FP64 pipe: their roofline is
+        # double arithmetic is bound by the FP64 pipe: the roofline is
         # max(HBM time, FP64-pipe instructions / measured FP64 issue rate),
         # the rate being the DGEMM peak over 2 flop per DFMA (a DADD or DMUL
-        # takes the pipe for the same slot as a DFMA)
+        # takes the pipe for the same slot as a DFMA); stages in fixed point
+        # execute none of these and count for nothing here
         ops = fp64_ops_record(name)
         pk = fp64_peak_tflops()
         out["fp64_peak_tflops"] = round(pk, 3)

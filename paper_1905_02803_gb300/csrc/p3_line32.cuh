@@ -15,8 +15,8 @@
 // Pass twiddles come from tables in the order that consecutive butterflies read
 // them (one sector per warp and value instead of up to one per lane).
 //
-// Measured (forward + inverse): 384^3 907 -> 689 us, 375 x 360 x 343 885 ->
-// 651 us, 24 mixed grids 2.49 -> 1.94 ms, 48 x 40 x 36 39 -> 25 us (replayed
+// Measured (forward + inverse): 384^3 907 -> 671 us, 375 x 360 x 343 885 ->
+// 645 us, 24 mixed grids 2.49 -> 1.75 ms, 48 x 40 x 36 37 -> 24 us (replayed
 // graph).  Per complex point a strided stage of 384 issues 80 instructions
 // (112 before), a row stage about 80 (125).  What bounds them now: no single
 // unit (L1 data pipe 41 - 64 % busy, issue about 50 %); the rest waits for the
