@@ -320,9 +320,14 @@ static p3_status batch_run(p3_batch b, int dir, const void* const* in, void* con
     }
     if (cur != b->device) return P3_ERR_INVALID;
     cudaStream_t s0 = (cudaStream_t)stream;
-    if (cudaEventRecord(b->fork, s0) != cudaSuccess) return P3_ERR_CUDA;
+    // a failed call's error does not stay behind for a later call to report
+    auto failed = [] {
+        cudaGetLastError();
+        return P3_ERR_CUDA;
+    };
+    if (cudaEventRecord(b->fork, s0) != cudaSuccess) return failed();
     for (cudaStream_t s : b->streams)
-        if (cudaStreamWaitEvent(s, b->fork, 0) != cudaSuccess) return P3_ERR_CUDA;
+        if (cudaStreamWaitEvent(s, b->fork, 0) != cudaSuccess) return failed();
     p3_status rc = P3_OK;
     for (size_t i = 0; i < n && rc == P3_OK; ++i)
         rc = p3::run_direction(b->plans[i], dir, in[i], out[i], ws ? ws[i] : NULL,
@@ -332,7 +337,7 @@ static p3_status batch_run(p3_batch b, int dir, const void* const* in, void* con
     for (size_t s = 0; s < b->streams.size(); ++s) {
         if (cudaEventRecord(b->join[s], b->streams[s]) != cudaSuccess ||
             cudaStreamWaitEvent(s0, b->join[s], 0) != cudaSuccess)
-            return P3_ERR_CUDA;
+            return failed();
     }
     return rc;
 }

@@ -1377,6 +1377,14 @@ static p3_status check_call(p3_plan P, int dir, const void* in, void* out, void*
     return P3_OK;
 }
 
+// A CUDA call of a transform failed: its error does not stay behind for a later
+// call of the library to take for its own.
+static p3_status cuda_failed()
+{
+    cudaGetLastError();
+    return P3_ERR_CUDA;
+}
+
 static p3_status run(p3_plan P, int dir, const void* in, void* out, void* ws, void* stream)
 {
     if (!P || !in || !out) return P3_ERR_INVALID;
@@ -1391,7 +1399,7 @@ static p3_status run(p3_plan P, int dir, const void* in, void* out, void* ws, vo
     cudaStream_t s = (cudaStream_t)stream;
     void* const bufs[3] = {const_cast<void*>(in), out, ws};
     cudaEvent_t* ev = P->timing ? (cudaEvent_t*)&P->events[dir * 4] : NULL;
-    if (ev && cudaEventRecord(ev[0], s) != cudaSuccess) return P3_ERR_CUDA;
+    if (ev && cudaEventRecord(ev[0], s) != cudaSuccess) return cuda_failed();
     int i = 0;
     for (auto& st : stages) {
         StageArgs a = st.a;
@@ -1417,15 +1425,15 @@ static p3_status run(p3_plan P, int dir, const void* in, void* out, void* ws, vo
             e = a.tma == 1 ? p3::pow2_encode_tma(a) : cudaSuccess;
             if (e == cudaSuccess) e = P->prec == P3_F32 ? p3::launch_stage_f32(a, s) : p3::launch_stage_f64(a, s);
         }
-        if (e != cudaSuccess) return P3_ERR_CUDA;
+        if (e != cudaSuccess) return cuda_failed();
         ++i;
         if (hook && (size_t)i == hook_after && call_hook(P, dir, a.dst, stream) != 0) return P3_ERR_HOOK;
-        if (ev && i <= 3 && cudaEventRecord(ev[i], s) != cudaSuccess) return P3_ERR_CUDA;
+        if (ev && i <= 3 && cudaEventRecord(ev[i], s) != cudaSuccess) return cuda_failed();
     }
     if (hook && stages.empty() && call_hook(P, dir, out, stream) != 0) return P3_ERR_HOOK;
     if (ev)
         for (int k = i + 1; k <= 3; ++k)
-            if (cudaEventRecord(ev[k], s) != cudaSuccess) return P3_ERR_CUDA;
+            if (cudaEventRecord(ev[k], s) != cudaSuccess) return cuda_failed();
     return P3_OK;
 }
 

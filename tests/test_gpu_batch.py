@@ -235,3 +235,38 @@ def test_streams_of_a_batch(grids, prec, asked, used):
     assert cu.cuGraphGetRootNodes(graph, None, ctypes.byref(count)) == 0
     assert count.value == used
     assert cu.cuGraphDestroy(graph) == 0
+
+
+@pytest.mark.parametrize("shape", [(30, 14, 9), (40, 1, 26), (64, 64, 64), (512, 256, 6)])
+def test_failed_launch_leaves_no_error_behind(shape):
+    """A call on a stream whose capture was invalidated fails on the host; the
+    next persistent batch call must not report that failure as its own."""
+    import ctypes
+
+    import torch
+    from paper_1905_02803_gb300 import p3dfft as P
+    cu = ctypes.CDLL("libcuda.so.1")
+    plan = P.Plan(*shape, precision="f32")
+    x = plan.empty_real().normal_()
+    X = plan.empty_complex()
+    batch = P.Batch([plan], nstreams=0)
+    ref = batch.forward([x])[0]
+    s = torch.cuda.Stream()
+    h = ctypes.c_void_p(s.cuda_stream)
+    graph = ctypes.c_void_p()
+    plan.workspace()
+    torch.cuda.synchronize()
+    assert cu.cuStreamBeginCapture_v2(h, 1) == 0
+    assert cu.cuStreamSynchronize(h) != 0  # not permitted: invalidates the capture
+    with pytest.raises(P.P3Error):
+        plan.forward(x, X, stream=s)
+    assert cu.cuStreamEndCapture(h, ctypes.byref(graph)) != 0
+    assert torch.equal(batch.forward([x])[0], ref)
+    # the same through a stream batch
+    streams = P.Batch([plan], nstreams=1)
+    assert cu.cuStreamBeginCapture_v2(h, 1) == 0
+    assert cu.cuStreamSynchronize(h) != 0
+    with torch.cuda.stream(s), pytest.raises(P.P3Error):
+        streams.forward([x], [X])
+    assert cu.cuStreamEndCapture(h, ctypes.byref(graph)) != 0
+    assert torch.equal(batch.forward([x])[0], ref)
